@@ -29,7 +29,10 @@ constexpr unsigned char kNo = 0, kYes = 1, kCodeFull = 2, kCodeReserved = 3;
 // Per-table counters and status, resident in device memory.
 //   I: non-empty cells (tombstones included), D: tombstones (Sec. 4.2/4.4).
 //   status: sticky kFull / kReserved bits.
-//   mig_fail: set by a migration CTA that could not bound its cluster range.
+//   mig_fail, mig_moved: set by a migration warp that could not bound its
+//   cluster range; live elements the migration has placed so far.  Both are
+//   zero between migrations (the last kernel of one clears them), so no
+//   memset precedes a migration.
 //   export_pos: output cursor of the export compaction.
 struct DevState {
     u64 I;
@@ -41,6 +44,7 @@ struct DevState {
     // (slot 0: key 0, slot 1: key ~0); untouched by migrations
     u64 sp_val[2];
     u32 sp_present[2];
+    u64 mig_moved;
 };
 
 // fmix64, the 64-bit finalizer of MurmurHash3 (Appleby, public domain).
@@ -92,6 +96,18 @@ __device__ __forceinline__ u64 ld_stream(const u64* p) {
 // 2-word CAS on a whole cell; returns the cell's previous content.
 __device__ __forceinline__ Cell cas_cell(Cell* p, Cell expect, Cell desired) {
     return atomicCAS(p, expect, desired);
+}
+
+// Programmatic dependent launch: the operation and
+// migration kernels are launched so that
+// the next one on the stream may be scheduled while this one drains; each
+// lets its dependents start at once and then waits until the grids before it
+// have completed and their memory is visible (a no-op when it was launched
+// the ordinary way).  Stream order of every memory effect is unchanged; the
+// launch latency of back-to-back calls overlaps the previous call's tail.
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace cht

@@ -11,14 +11,12 @@
 // an operation round of min(floor(alpha * c) - I, rest) operations, so I never
 // passes the threshold (the same chunks the host-driven policy makes).  Every
 // warp of the grid then works on the round: operation pieces from a ticket
-// counter with the group probe loop, or the migration's tile borders, a
-// barrier, and the tile placement (the same device code as the migration
-// kernels).  The barriers replace the host's counter read-back and the
+// counter with the group probe loop, or the migration's tiles (the same
+// device code as the migration kernels).  The barriers replace the host's counter read-back and the
 // launches between rounds.
 //
 // Memory.  The host allocates two target tables of the largest capacity the
-// batch can need (every operation a new key) and the border scratch; the table
-// moves initial cells -> target 1 -> target 2 -> target 1 ... and the host
+// batch can need (every operation a new key); the table moves initial cells -> target 1 -> target 2 -> target 1 ... and the host
 // frees what is not the final table after the launch.
 //
 // Bounded waits.  A barrier wait gives up after `spin_limit` clock cycles: the
@@ -44,7 +42,6 @@ struct GrowArgs {
     u32 max_log2;     // capacity of the targets
     double alpha;
     GrowCtl* ctl;
-    u64* border;      // tile borders of the largest source
     long long spin_limit;
     int stall_block;  // testing: this block never arrives at a barrier (-1: none)
 };
@@ -151,7 +148,7 @@ __global__ void __launch_bounds__(kGrowBlock) grow_kernel(GrowArgs g) {
             if (leader) c->done = done + chunk;
             continue;
         }
-        // migration round: borders, then placement (Sec. 4.3.1)
+        // migration round (Sec. 4.3.1)
         const u32 tgt = cur == 1u ? 2u : 1u;
         MigArgs m;
         m.src = g.tab[cur];
@@ -159,17 +156,9 @@ __global__ void __launch_bounds__(kGrowBlock) grow_kernel(GrowArgs g) {
         m.dst = g.tab[tgt];
         m.dlog2 = *reinterpret_cast<volatile unsigned int*>(&c->next_log2);
         m.st = st;
-        m.border = g.border;
         m.tile = (1ull << log2c) < kGrowTile ? u32(1ull << log2c) : kGrowTile;
         const bool windows = *reinterpret_cast<volatile unsigned int*>(&c->windows) != 0;
         m.start_cap = migrate_start_cap(m.tile, windows);
-        migrate_borders<true>(m, u64(blockIdx.x) * kGrowBlock + threadIdx.x, u64(gridDim.x) * kGrowBlock);
-        if (leader) {  // the kernels below accumulate the moved elements into I
-            st->I = 0;
-            st->D = 0;
-            st->mig_fail = 0;
-        }
-        if (!grid_sync(g, gen)) return;
         if (windows) migrate_window_tiles<true>(m, smem, warp, nwarps);
         else migrate_walk_tiles<true>(m, smem, warp, nwarps);
         if (!grid_sync(g, gen)) return;
@@ -180,11 +169,15 @@ __global__ void __launch_bounds__(kGrowBlock) grow_kernel(GrowArgs g) {
                 atomicOr(&c->error, kGrowMigFail);
                 c->fail_tgt = tgt;
                 c->action = kActDone;
+                st->mig_fail = 0;
             } else {
+                st->I = *reinterpret_cast<volatile unsigned long long*>(&st->mig_moved);
+                st->D = 0;
                 c->cur = tgt;
                 c->log2c = m.dlog2;
                 ++c->migrations;
             }
+            st->mig_moved = 0;
         }
         if (!grid_sync(g, gen)) return;
         if (*reinterpret_cast<volatile unsigned int*>(&c->error)) return;
@@ -217,11 +210,8 @@ cudaError_t launch_mode(const GrowArgs& g, int group_width, int lane_cells, cuda
 
 }  // namespace
 
-// a purge (gamma = 1) at the largest capacity migrates a source of max_log2
-u64 grow_border_count(u32 max_log2) { return migrate_border_count(max_log2, kGrowTile); }
-
 cudaError_t launch_grow(const OpArgs& op, Mode mode, Cell* t1, Cell* t2, u32 max_log2, double alpha, GrowCtl* ctl,
-                        u64* border, long long spin_limit, int stall_block, int group_width, cudaStream_t s) {
+                        long long spin_limit, int stall_block, int group_width, cudaStream_t s) {
     GrowArgs g;
     g.op = op;
     g.tab[0] = op.cells;
@@ -230,7 +220,6 @@ cudaError_t launch_grow(const OpArgs& op, Mode mode, Cell* t1, Cell* t2, u32 max
     g.max_log2 = max_log2;
     g.alpha = alpha;
     g.ctl = ctl;
-    g.border = border;
     g.spin_limit = spin_limit;
     g.stall_block = stall_block;
     switch (mode) {

@@ -57,14 +57,12 @@ cudaError_t launch_iou_aggregated_wide(Mode mode, const OpArgs& a, bool warp_ded
 
 // Cluster-wise migration of `src` (2^src_log2 cells) into `dst`
 // (2^dst_log2 cells, dst_log2 >= src_log2).  dst needs no initialisation:
-// every target cell is written.  `st` receives the new I (it must be zero
-// on entry) and mig_fail.  tile: source cells per warp task (power of two,
-// 0 = default); windows: place cells 32 at a time per warp (long clusters)
-// instead of one cluster per lane; border: device scratch of
-// migrate_border_count() u64.
-u64 migrate_border_count(u32 src_log2, int tile);
+// every target cell is written.  `st` receives the new I and D = 0.  tile:
+// source cells per warp task (power of two, 0 = default); windows: place
+// cells 32 at a time per warp (long clusters) instead of one cluster per
+// lane.
 cudaError_t launch_migrate(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log2, DevState* st,
-                           int tile, bool windows, u64* border, cudaStream_t s);
+                           int tile, bool windows, cudaStream_t s);
 
 // Shrinking migration (Sec. 4.3.1 "Shrinking") of `src` into `dst` (2^dst_log2
 // cells, dst_log2 < src_log2, more cells than live elements; no
@@ -159,10 +157,9 @@ struct GrowCtl {
     unsigned long long chunk;   // operations of the current round
     unsigned long long ticket;  // pieces taken in the current round
 };
-u64 grow_border_count(u32 max_log2);
 // group_width 1 (one lane per key, one sector per lane) or 4 (four lanes x one sector).
 cudaError_t launch_grow(const OpArgs& op, Mode mode, Cell* t1, Cell* t2, u32 max_log2, double alpha, GrowCtl* ctl,
-                        u64* border, long long spin_limit, int stall_block, int group_width, cudaStream_t s);
+                        long long spin_limit, int stall_block, int group_width, cudaStream_t s);
 
 // Compact the live cells into keys_out / vals_out (max_n entries); the count
 // lands in st->export_pos, which must be zero on entry.

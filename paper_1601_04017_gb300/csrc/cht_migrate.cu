@@ -15,10 +15,9 @@
 // live cells are re-inserted in source index order, so the layout equals the
 // sequential migration (Lemma 1).
 //
-// GB300 mapping.  A border kernel computes m(d) for every tile once (a short
-// forward scan per tile).  In the migration kernel every warp then works on
-// its own tiles with no block-wide barrier, so a long cluster only delays
-// its own warp.  The warp reads its source range coalesced, 32 cells per
+// GB300 mapping.  Every warp works on its own tiles with no block-wide
+// barrier, so a long cluster only delays its own warp; it finds the tile's two
+// moved borders by a short forward scan each (warp_border).  The warp reads its source range coalesced, 32 cells per
 // window with the next 64 in flight, and re-inserts the window's live cells
 // in source order: all lanes look up the first free target cell at or after
 // their new home at once, and rounds of warp votes settle lanes that picked
@@ -30,35 +29,43 @@
 // 32-byte sector once and whole; longer ranges store elements directly and
 // zero-fill the rest.
 // A border scan that finds no empty cell within kMaxScan cells (a full
-// table, or a cluster longer than that) sets mig_fail; a single-CTA fallback
-// kernel, always launched after the tile kernel, then redoes the whole
-// migration sequentially.
+// table, or a cluster longer than that) sets mig_fail; a single-CTA kernel,
+// always launched after the tile kernel, sets the counters and, if mig_fail
+// is set, first redoes the whole migration sequentially.
+#include <atomic>
+
 #include "cht_migrate.cuh"
 
 namespace cht {
 namespace {
 
-// The kernels of a host-driven migration: one thread per tile for the
-// borders, then one warp per tile (in turn) for the placement.
-__global__ void __launch_bounds__(256) migrate_border_kernel(MigArgs a) {
-    migrate_borders(a, u64(blockIdx.x) * blockDim.x + threadIdx.x, u64(gridDim.x) * blockDim.x);
-}
-
+// The kernels of a host-driven migration: one warp per tile (in turn).
 __global__ void __launch_bounds__(kMigBlock, 5) migrate_window_kernel(MigArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pdl_enter();
     migrate_window_tiles(a, smem, u64(blockIdx.x) * kMigWarps + (threadIdx.x >> 5), u64(gridDim.x) * kMigWarps);
 }
 
 __global__ void __launch_bounds__(kMigBlock, 5) migrate_walk_kernel(MigArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pdl_enter();
     migrate_walk_tiles(a, smem, u64(blockIdx.x) * kMigWarps + (threadIdx.x >> 5), u64(gridDim.x) * kMigWarps);
 }
 
-// Sequential migration of the whole table by one thread (after a block-wide
-// zero fill), used only when a tile CTA reported mig_fail.  Visits the source
-// in index order from the first cluster start (index 0 if there is none).
-__global__ void __launch_bounds__(kMigBlock) migrate_fallback_kernel(MigArgs a) {
-    if (a.st->mig_fail == 0) return;
+// The end of a migration: I = the elements moved, D = 0.  If a tile's warp
+// reported mig_fail, the whole table is first migrated again, sequentially by
+// one thread (after a block-wide zero fill), visiting the source in index
+// order from the first cluster start (index 0 if there is none).
+__global__ void __launch_bounds__(kMigBlock) migrate_finish_kernel(MigArgs a) {
+    pdl_enter();
+    if (a.st->mig_fail == 0) {
+        if (threadIdx.x == 0) {
+            a.st->I = a.st->mig_moved;
+            a.st->D = 0;
+            a.st->mig_moved = 0;
+        }
+        return;
+    }
     const u64 c = 1ull << a.slog2, cmask = c - 1;
     const u64 nc = 1ull << a.dlog2, nmask = nc - 1;
     const u32 dshift = 64u - a.dlog2;
@@ -87,15 +94,14 @@ __global__ void __launch_bounds__(kMigBlock) migrate_fallback_kernel(MigArgs a) 
             p = (p + 1) & nmask;
             ++steps;
         }
-        if (steps >= nc) {
-            a.st->mig_fail = 4u;  // target too small: cannot happen for gamma >= 1
-            return;
-        }
+        if (steps >= nc) break;  // target too small: cannot happen for gamma >= 1
         a.dst[p] = cl;
         ++moved;
     }
     a.st->I = moved;
-    a.st->mig_fail = 8u;  // fallback ran and completed
+    a.st->D = 0;
+    a.st->mig_moved = 0;
+    a.st->mig_fail = 0;
 }
 
 __global__ void __launch_bounds__(256) export_kernel(const Cell* __restrict__ cells, u64 c,
@@ -291,15 +297,49 @@ cudaError_t launch_shrink(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log2
     return cudaGetLastError();
 }
 
-u64 migrate_border_count(u32 src_log2, int tile) {
-    const u64 c = 1ull << src_log2;
-    u64 T = tile > 0 ? u64(tile) : 256u;
-    if (T > c) T = c;
-    return c / T;
+namespace {
+
+// Launch with programmatic stream serialization (see pdl_enter).
+template <typename K>
+cudaError_t launch_pdl(K kernel, unsigned grid, size_t smem, cudaStream_t s, const MigArgs& a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kMigBlock);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// Resident CTAs per SM of a migration kernel with its shared memory for
+// `start_cap` (asked once per kernel and tile size, not per migration).
+cudaError_t resident_ctas(bool windows, u32 tile_log2, size_t smem, int* per_sm) {
+    static std::atomic<int> known[2][16];
+    std::atomic<int>& k = known[windows ? 1 : 0][tile_log2 & 15u];
+    *per_sm = k.load(std::memory_order_relaxed);
+    if (*per_sm > 0) return cudaSuccess;
+    const void* fn = windows ? reinterpret_cast<const void*>(migrate_window_kernel)
+                             : reinterpret_cast<const void*>(migrate_walk_kernel);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(migrate_smem_bytes(migrate_start_cap(8192, windows))));
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, kMigBlock, smem);
+    if (e != cudaSuccess) return e;
+    if (*per_sm < 1) *per_sm = 1;
+    k.store(*per_sm, std::memory_order_relaxed);
+    return cudaSuccess;
+}
+
+}  // namespace
+
 cudaError_t launch_migrate(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log2, DevState* st,
-                           int tile, bool windows, u64* border, cudaStream_t s) {
+                           int tile, bool windows, cudaStream_t s) {
     const u64 c = 1ull << src_log2;
     u32 T = tile > 0 ? u32(tile) : 256u;
     if (T > c) T = u32(c);
@@ -309,39 +349,22 @@ cudaError_t launch_migrate(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log
     a.dst = dst;
     a.dlog2 = dst_log2;
     a.st = st;
-    a.border = border;
     a.tile = T;
     a.start_cap = migrate_start_cap(T, windows);
     const u64 ntiles = c / T;
-    u64 bgrid = (ntiles + 255) / 256;
-    const u64 bcap = u64(sm_count()) * 8;
-    if (bgrid > bcap) bgrid = bcap;
-    migrate_border_kernel<<<unsigned(bgrid), 256, 0, s>>>(a);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    u32 tlog2 = 0;
+    while ((1u << tlog2) < T) ++tlog2;
     const size_t smem = migrate_smem_bytes(a.start_cap);
-    const void* fn = windows ? reinterpret_cast<const void*>(migrate_window_kernel)
-                             : reinterpret_cast<const void*>(migrate_walk_kernel);
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kMigBlock, smem);
+    cudaError_t e = resident_ctas(windows, tlog2, smem, &per_sm);
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     u64 grid = u64(sm_count()) * per_sm;
     const u64 need = (ntiles + kMigWarps - 1) / kMigWarps;
     if (grid > need) grid = need;
-    if (windows)
-        migrate_window_kernel<<<unsigned(grid), kMigBlock, smem, s>>>(a);
-    else
-        migrate_walk_kernel<<<unsigned(grid), kMigBlock, smem, s>>>(a);
-    count_launch();
-    e = cudaGetLastError();
+    e = windows ? launch_pdl(migrate_window_kernel, unsigned(grid), smem, s, a)
+                : launch_pdl(migrate_walk_kernel, unsigned(grid), smem, s, a);
     if (e != cudaSuccess) return e;
-    migrate_fallback_kernel<<<1, kMigBlock, 0, s>>>(a);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(migrate_finish_kernel, 1, 0, s, a);
 }
 
 cudaError_t launch_export(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, u64 max_n,

@@ -23,7 +23,6 @@ struct MigArgs {
     Cell* dst;
     u32 dlog2;
     DevState* st;
-    u64* border;     // m(d) of every tile (scratch, ntiles entries)
     u32 tile;        // T, power of two, <= c
     u32 start_cap;   // per-warp capacity of the cluster-start list (walk kernel)
 };
@@ -58,30 +57,24 @@ __device__ __forceinline__ void src_pair(const Cell* p, u64& k0, u64& v0, u64& k
     else ld_pair_nc(p, k0, v0, k1, v1);
 }
 
-// m(d) for every tile: d itself if cell d-1 is empty, else one past the
-// first empty cell >= d (unwrapped: may exceed c for the last tiles).
-// Threads first, first + stride, ... each take tiles in turn.
+// m(d) of a tile border d: d itself if cell d-1 is empty, else one past the
+// first empty cell >= d (unwrapped: may exceed c for the last tiles), by the
+// whole warp, 32 cells a step; kNoBorder if there is none within kMaxScan
+// cells.  Every tile's warp finds both its borders itself: the neighbours'
+// warps scan the same few cells again (1.5 to 50 of them on average at loads
+// 0.5 to 0.9), which costs less than a launch of its own, its scratch array
+// and the wait between the two (4-9 us of a 40-60 us migration of 2^12-2^20
+// cells).
 template <bool kCg = false>
-__device__ __forceinline__ void migrate_borders(const MigArgs& a, u64 first, u64 stride) {
+__device__ __forceinline__ u64 warp_border(const MigArgs& a, u64 d, int lane) {
     const u64 c = 1ull << a.slog2, cmask = c - 1;
-    const u64 ntiles = c / a.tile;
-    for (u64 t = first; t < ntiles; t += stride) {
-        const u64 d = t * a.tile;
-        u64 m = kNoBorder;
-        if (src_key<kCg>(a.src + ((d - 1) & cmask)) == kEmpty) {
-            m = d;
-        } else {
-            const u64 lim = c < kMaxScan ? c : kMaxScan;
-            for (u64 i = d; i < d + lim; i += 2) {
-                u64 k0, v0, k1, v1;
-                src_pair<kCg>(a.src + (i & cmask), k0, v0, k1, v1);  // d is even: pairs stay aligned
-                if (k0 == kEmpty) { m = i + 1; break; }
-                if (k1 == kEmpty) { m = i + 2; break; }
-            }
-        }
-        if (m == kNoBorder) atomicOr(&a.st->mig_fail, 1u);
-        a.border[t] = m;
+    if (src_key<kCg>(a.src + ((d - 1) & cmask)) == kEmpty) return d;
+    const u64 lim = c < kMaxScan ? c : kMaxScan;
+    for (u64 i = 0; i < lim; i += 32) {
+        const u32 e = __ballot_sync(0xffffffffu, src_key<kCg>(a.src + ((d + i + lane) & cmask)) == kEmpty);
+        if (e) return d + i + u64(__ffs(e));
     }
+    return kNoBorder;
 }
 
 __device__ __forceinline__ u64 warp_sum(u64 x) {
@@ -276,11 +269,15 @@ struct Tile {
     int mode;
 };
 
-__device__ __forceinline__ bool tile_of(const MigArgs& a, u64 t, u64 ntiles, Tile& x) {
+template <bool kCg = false>
+__device__ __forceinline__ bool tile_of(const MigArgs& a, u64 t, u64 ntiles, Tile& x, int lane) {
     const u64 c = 1ull << a.slog2;
-    const u64 m0 = a.border[t];
-    const u64 b1 = t + 1 < ntiles ? a.border[t + 1] : a.border[0];
-    if (m0 == kNoBorder || b1 == kNoBorder) return false;  // fallback redoes everything
+    const u64 m0 = warp_border<kCg>(a, t * a.tile, lane);
+    const u64 b1 = warp_border<kCg>(a, t + 1 < ntiles ? (t + 1) * a.tile : 0, lane);
+    if (m0 == kNoBorder || b1 == kNoBorder) {  // the fallback redoes everything
+        if (lane == 0) atomicOr(&a.st->mig_fail, 1u);
+        return false;
+    }
     const u64 m1 = t + 1 < ntiles ? b1 : b1 + c;
     if (m1 <= m0) return false;  // the tile lies inside a cluster owned by an earlier tile
     const u32 g = a.dlog2 - a.slog2;
@@ -359,7 +356,7 @@ __device__ __forceinline__ void migrate_window_tiles(const MigArgs& a, unsigned 
     bool bad = false;
     for (u64 t = warp; t < ntiles && !bad; t += nwarps) {
         Tile x;
-        if (!tile_of(a, t, ntiles, x)) continue;
+        if (!tile_of<kCg>(a, t, ntiles, x, lane)) continue;
         u32* const bm = x.mode == 0 ? small_bm : region;
         clear_owned(a, x, bm, lane);
         if (x.mode == 0)
@@ -373,7 +370,7 @@ __device__ __forceinline__ void migrate_window_tiles(const MigArgs& a, unsigned 
     }
     if (bad && lane == 0) atomicOr(&a.st->mig_fail, 2u);
     moved = warp_sum(moved);
-    if (lane == 0 && moved) atomicAdd(&a.st->I, moved);
+    if (lane == 0 && moved) atomicAdd(&a.st->mig_moved, moved);
 }
 
 // Migration by clusters (tables below load 0.6, where clusters are short and
@@ -403,7 +400,7 @@ __device__ __forceinline__ void migrate_walk_tiles(const MigArgs& a, unsigned ch
 
     for (u64 t = warp; t < ntiles; t += nwarps) {
         Tile x;
-        if (!tile_of(a, t, ntiles, x)) continue;
+        if (!tile_of<kCg>(a, t, ntiles, x, lane)) continue;
         u32* const bm = x.mode == 0 ? small_bm : region;
         clear_owned(a, x, bm, lane);
 
@@ -491,7 +488,7 @@ __device__ __forceinline__ void migrate_walk_tiles(const MigArgs& a, unsigned ch
     }
     if (bad && lane == 0) atomicOr(&a.st->mig_fail, 2u);
     moved = warp_sum(moved);
-    if (lane == 0 && moved) atomicAdd(&a.st->I, moved);
+    if (lane == 0 && moved) atomicAdd(&a.st->mig_moved, moved);
 }
 
 // Shared memory of the tile loops for one 256-thread block.

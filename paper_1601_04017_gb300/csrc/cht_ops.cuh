@@ -571,17 +571,6 @@ constexpr int op_min_blocks() {
     return (V == 4 && G >= 4) ? 5 : 1;
 }
 
-// Programmatic dependent launch: the operation kernels are launched so that
-// the next one on the stream may be scheduled while this one drains; each
-// lets its dependents start at once and then waits until the grids before it
-// have completed and their memory is visible (a no-op when it was launched
-// the ordinary way).  Stream order of every memory effect is unchanged; the
-// launch latency of back-to-back calls overlaps the previous call's tail.
-__device__ __forceinline__ void pdl_enter() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 template <int G, int V, int MODE, int kFlags>
 __global__ void __launch_bounds__(kOpBlock, op_min_blocks<G, V>()) op_kernel(OpArgs a) {
     pdl_enter();

@@ -247,6 +247,12 @@ cht_status read_state(cht_table* h, DevState* out, cudaStream_t s) {
     return cuda_status(cudaStreamSynchronize(s));
 }
 
+// Tables too small to give every warp task slot of the GPU (152 SMs x 5 CTAs
+// x 8 warps = 6080) a tile of the usual size are cut finer, down to 64 cells:
+// a tile is one warp's serial work, and a migration of 2^12..2^20 cells takes
+// about one tile's time.
+constexpr u64 kMigTasks = 4096;
+
 // Migrate h into 2^new_log2 cells (new_log2 >= log2c).  `live` is the exact
 // live count if known (else ~0).  Allocates first: on failure h is unchanged.
 cht_status do_migrate(cht_table* h, u32 new_log2, u64 live, cudaStream_t s) {
@@ -258,35 +264,36 @@ cht_status do_migrate(cht_table* h, u32 new_log2, u64 live, cudaStream_t s) {
     const u64 bytes = (1ull << new_log2) * sizeof(Cell);
     cht_status r = lib_alloc(reinterpret_cast<void**>(&dst), bytes, s);
     if (r != CHT_OK) return r;
-    // below load 0.6 (short clusters) one lane re-inserts each cluster; above
-    // it (long clusters) the warp places 32 cells at a time.  Tiles of 512 and
-    // 1024 cells were the fastest of 256..2048 for each (2^28 cells, GB300).
-    const bool windows = double(h->i_bound) >= 0.6 * double(h->cap());
-    int tile = h->cfg.migrate_tile;
-    if (tile == 0) tile = windows ? 1024 : 512;
-    // scratch: the moved border of every migration tile (growing), or the
-    // spill list of c' cells plus its counter (shrinking)
-    const u64 sbytes = shrink ? bytes + 256 : cht::migrate_border_count(h->log2c, tile) * sizeof(u64);
-    unsigned char* scratch = nullptr;
-    r = lib_alloc(reinterpret_cast<void**>(&scratch), sbytes, s);
-    if (r != CHT_OK) {
-        lib_free(dst, bytes, s);
-        return r;
-    }
-    // I and D restart (the kernels accumulate the moved count into I)
-    cudaError_t e = cudaMemsetAsync(&h->st->I, 0, 2 * sizeof(u64), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&h->st->mig_fail, 0, sizeof(u32), s);
+    cudaError_t e = cudaSuccess;
     if (shrink) {
+        // scratch: the spill list of c' cells plus its counter
+        const u64 sbytes = bytes + 256;
+        unsigned char* scratch = nullptr;
+        r = lib_alloc(reinterpret_cast<void**>(&scratch), sbytes, s);
+        if (r != CHT_OK) {
+            lib_free(dst, bytes, s);
+            return r;
+        }
         unsigned long long* nspill = reinterpret_cast<unsigned long long*>(scratch + bytes);
+        // I and D restart (the kernels accumulate the moved count into I)
+        e = cudaMemsetAsync(&h->st->I, 0, 2 * sizeof(u64), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(nspill, 0, sizeof(unsigned long long), s);
         if (e == cudaSuccess)
             e = cht::launch_shrink(h->cells, h->log2c, dst, new_log2, h->st, reinterpret_cast<Cell*>(scratch),
                                    nspill, s);
-    } else if (e == cudaSuccess) {
-        e = cht::launch_migrate(h->cells, h->log2c, dst, new_log2, h->st, tile, windows,
-                                reinterpret_cast<u64*>(scratch), s);
+        lib_free(scratch, sbytes, s);
+    } else {
+        // below load 0.6 (short clusters) one lane re-inserts each cluster; above
+        // it (long clusters) the warp places 32 cells at a time.  Tiles of 512 and
+        // 1024 cells were the fastest of 256..2048 for each (2^28 cells, GB300).
+        const bool windows = double(h->i_bound) >= 0.6 * double(h->cap());
+        int tile = h->cfg.migrate_tile;
+        if (tile == 0) {
+            tile = windows ? 1024 : 512;
+            while (tile > 64 && (h->cap() / u64(tile)) < kMigTasks) tile /= 2;
+        }
+        e = cht::launch_migrate(h->cells, h->log2c, dst, new_log2, h->st, tile, windows, s);
     }
-    lib_free(scratch, sbytes, s);
     if (e != cudaSuccess) {
         lib_free(dst, bytes, s);
         return cuda_status(e);
@@ -474,18 +481,14 @@ cht_status grow_in_kernel(cht_table* h, cht::Mode mode, const u64* keys, const u
     u32 ml = h->log2c;
     while (ml < kMaxLog2 && u64(std::floor(alpha * double(1ull << ml))) < bound) ++ml;
     const u64 tbytes = (1ull << ml) * sizeof(Cell);
-    const u64 bbytes = cht::grow_border_count(ml) * sizeof(u64);
     Cell *t1 = nullptr, *t2 = nullptr;
-    u64* border = nullptr;
     cht::GrowCtl* ctl = nullptr;
     cht_status r = lib_alloc(reinterpret_cast<void**>(&t1), tbytes, s);
     if (r == CHT_OK) r = lib_alloc(reinterpret_cast<void**>(&t2), tbytes, s);
-    if (r == CHT_OK) r = lib_alloc(reinterpret_cast<void**>(&border), bbytes, s);
     if (r == CHT_OK) r = lib_alloc(reinterpret_cast<void**>(&ctl), sizeof(cht::GrowCtl), s);
     auto release = [&]() {
         lib_free(t1, tbytes, s);
         lib_free(t2, tbytes, s);
-        lib_free(border, bbytes, s);
         lib_free(ctl, sizeof(cht::GrowCtl), s);
     };
     if (r != CHT_OK) {
@@ -511,7 +514,7 @@ cht_status grow_in_kernel(cht_table* h, cht::Mode mode, const u64* keys, const u
     const long long spin = (h->cfg.grow_spin_us > 0 ? (long long)h->cfg.grow_spin_us : 1000000ll) * 2100;  // ~2.1 GHz
     cudaError_t e = cudaMemcpyAsync(ctl, &init, sizeof(init), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = cht::launch_grow(a, mode, t1, t2, ml, alpha, ctl, border, spin, h->cfg.grow_fault_inject ? 1 : -1,
+        e = cht::launch_grow(a, mode, t1, t2, ml, alpha, ctl, spin, h->cfg.grow_fault_inject ? 1 : -1,
                              w.g == 1 ? 1 : 4, s);
     cht::GrowCtl fin;
     DevState ds;
