@@ -190,6 +190,23 @@ __device__ __forceinline__ void op_vout(const OpArgs& a, const WarpStage& sg, u6
 constexpr int kFlagReuse = 1;
 constexpr int kFlagFullKeys = 2;
 
+// Results of finds with one-line windows on HBM-sized tables.  Such a find is
+// bound by the L2 requests it makes (random lines: ~47 G requests a second,
+// loads and stores alike), and the groups of a warp finish out of order, so
+// storing each result as it comes made one request per ~3 results (57 M for
+// 2^25 finds, of which ~38 M are the lines probed).  The warp therefore keeps
+// its results in a ring of kRingOps operations in shared memory and writes
+// them in order, 32 at a time, once the window behind them is used up; an
+// operation still probing then stores its own result.  2^25 finds on 2^26
+// cells: 1037 -> 978 us at load 0.5, 1316 -> 1231 us at load 0.7.  (Wider
+// windows make many requests per find and spill with the ring's registers.)
+constexpr u32 kRingOps = 128;             // the windows in use, the one before, and as many to spare
+constexpr unsigned char kPending = 0xff;  // no result yet
+template <int G, int V, int MODE, bool kCoherent, bool kStaged, int kFlags>
+constexpr bool use_ring() {
+    return MODE == kFind && !kCoherent && !kStaged && kFlags == 0 && G * V * int(sizeof(Cell)) <= 128;
+}
+
 template <int G, int V, int MODE, bool kCoherent = false, bool kStaged = false, int kFlags = 0>
 __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 end, u64& n_ins, u64& n_del,
                                          u32& sbits, const WarpStage& sg = WarpStage{}) {
@@ -209,6 +226,18 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
     // spilled more registers and the load-0.9 inserts took 10.2 -> 14.4 ms;
     // one-line windows gain nothing, the line is fetched whole anyway.)
     constexpr bool kSkipBeforeFirst = MODE == kFind && W * sizeof(Cell) > 128;
+    // Finds with one-line windows keep their results in the warp's part of a
+    // shared ring and write them 32 operations at a time.
+    constexpr bool kRing = use_ring<G, V, MODE, kCoherent, kStaged, kFlags>();
+    __shared__ u64 s_rv[kRing ? kOpBlock / 32 : 1][kRing ? kRingOps : 1];
+    __shared__ unsigned char s_rc[kRing ? kOpBlock / 32 : 1][kRing ? kRingOps : 1];
+    u64* const rv = s_rv[kRing ? threadIdx.x >> 5 : 0];
+    unsigned char* const rc = s_rc[kRing ? threadIdx.x >> 5 : 0];
+    u64 flushed = next;  // operations below it are written, or write themselves
+    if (kRing) {
+        for (u32 j = threadIdx.x & 31; j < kRingOps; j += 32) rc[j] = kPending;
+        __syncwarp();
+    }
 
     const u64 cap = 1ull << a.log2c;
     const u64 cmask = cap - 1;
@@ -245,6 +274,31 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
         }
     }
 
+    auto put = [&](u64 i, u64 v, unsigned char c) {  // a find's result
+        if (kRing && i >= flushed) {
+            rv[i & (kRingOps - 1)] = v;
+            rc[i & (kRingOps - 1)] = c;
+        } else {
+            op_vout<kStaged>(a, sg, i, v);
+            op_code<kStaged>(a, sg, i, c);
+        }
+    };
+    auto flush = [&](u64 upto) {  // the next 32 results, below `upto`
+        __syncwarp();
+        const u64 i = flushed + lane;
+        if (i < upto) {
+            const u32 j = u32(i) & (kRingOps - 1);
+            const unsigned char c = rc[j];
+            if (c != kPending) {
+                a.vals_out[i] = rv[j];
+                if (a.codes) a.codes[i] = c;
+                rc[j] = kPending;
+            }
+        }
+        flushed += 32;
+        __syncwarp();
+    };
+
     for (;;) {
         // ---- refill idle groups from this warp's slice
         bool fresh = false;
@@ -272,9 +326,10 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
                                 u64 v = 0;
                                 op_code<kStaged>(a, sg, idx, special_op<MODE>(a.st, key, d, &v));
                                 if (MODE == kFind) op_vout<kStaged>(a, sg, idx, v);
+                            } else if (MODE == kFind) {
+                                put(idx, 0, kCodeReserved);
                             } else {
                                 op_code<kStaged>(a, sg, idx, kCodeReserved);
-                                if (MODE == kFind) op_vout<kStaged>(a, sg, idx, 0);
                             }
                         }
                         if (!kFullKeys) sbits |= kReserved;
@@ -290,6 +345,9 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
             next += __popc(idle);
             if (!kStaged && next - wbase >= 32) {  // slide: nxt becomes cur, load the one after
                 wbase += 32;
+                // (the window before the one just used up: its last probes
+                // have had at least one step)
+                if (kRing && wbase - flushed >= 64) flush(end);
                 k_cur = k_nxt;
                 v_cur = v_nxt;
                 if (wbase + 32 + lane < end) {
@@ -438,10 +496,7 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
         int outcome = kStepContinue;
         if (active && ghit >= 0) {
             if (MODE == kFind) {
-                if (gl == 0) {
-                    op_vout<kStaged>(a, sg, idx, gmatch ? gval : 0);
-                    op_code<kStaged>(a, sg, idx, gmatch ? kYes : kNo);
-                }
+                if (gl == 0) put(idx, gmatch ? gval : 0, gmatch ? kYes : kNo);
                 active = false;
             } else if (gl == 0) {
                 if (kInsLike && !gmatch && tdist != 0)
@@ -498,8 +553,7 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
                 // every cell was examined without a decision
                 if (gl == 0) {
                     if (MODE == kFind) {
-                        op_vout<kStaged>(a, sg, idx, 0);
-                        op_code<kStaged>(a, sg, idx, kNo);
+                        put(idx, 0, kNo);
                     } else if (MODE == kErase || kUpdate) {
                         op_code<kStaged>(a, sg, idx, kNo);
                     } else {
@@ -511,7 +565,8 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
             }
         }
     }
-
+    if (kRing)
+        while (flushed < end) flush(end);
 }
 
 // Sum the CTA's counters and status bits into the table's device state with
