@@ -300,6 +300,7 @@ struct PlaceArgs {
     u32* deferred;         // cells whose survivor test was deferred (count in ex->n_deferred)
     unsigned char* dirty;  // per chunk: a deferred cell of it turned out to survive
     Cell* cells;           // the table
+    int dense;             // write every cell of the table, empty ones too
     Cell* ov;              // survivors past the last cell, by rank
     BuildExtra* ex;
 };
@@ -320,11 +321,11 @@ constexpr int kRunScan = 32;  // cells a survivor test looks ahead before deferr
 // test is deferred (2) to a CTA of its own (build_resolve_kernel), so that a
 // rare key inside a long run of copies of another key costs no long scan by
 // one thread.
-__device__ __forceinline__ unsigned char survivor_first(const PlaceArgs& a, u64 i, u64 k, u64 kn) {
+// k, s: the cell's key and sort key; kn, sn: the next cell's.
+__device__ __forceinline__ unsigned char survivor_first(const PlaceArgs& a, u64 i, u64 k, u64 s, u64 kn, u64 sn) {
     if (is_reserved(k)) return 0;
     if (i + 1 >= a.n) return 1;
-    const u64 s = sort_key(k, a.B);
-    if (sort_key(kn, a.B) != s) return 1;
+    if (sn != s) return 1;
     if (kn == k) return 0;
     for (u64 j = i + 2; j < a.n && j < i + 2 + kRunScan; ++j) {
         const u64 kj = ld_key(a.srt + j);
@@ -336,51 +337,113 @@ __device__ __forceinline__ unsigned char survivor_first(const PlaceArgs& a, u64 
 
 // Count passes (MODE 0: decide survivors and write the flags; MODE 1: only
 // for chunks where a deferred cell survived, recount from the flags) and the
-// write pass
-// (MODE 2).  Each thread takes kPlaceItems consecutive sorted cells.  The
-// count passes store each chunk's join; the write pass turns the chunk's
-// exclusive prefix plus the thread's into ranks and positions.
+// write pass (MODE 2).  Each thread takes kPlaceItems consecutive sorted
+// cells.  The count passes store each chunk's join; the write pass turns the
+// chunk's exclusive prefix plus the thread's into ranks and positions.
+//
+// The chunk goes through shared memory: coalesced loads in, and each thread
+// reads its consecutive cells from there, one slot of padding after every
+// kPlaceItems so that the threads of a warp fall on different banks.  (Loaded
+// by their threads directly, every load instruction touched 32 lines, and the
+// unpadded stage had 8-way bank conflicts on every store: the write pass was
+// bound by shared memory, short_scoreboard 12 per issue.  2^25 cells into
+// 2^26: count 170 -> 134 us, write 382 -> 313 us.)
+__device__ __forceinline__ u32 padded(u32 i) { return i + i / kPlaceItems; }
+constexpr u32 kPlaceWin = 2048;  // cells per window of a dense write
+constexpr u32 kPlacePad = kPlaceChunk + kPlaceChunk / kPlaceItems;
+
 template <int MODE>
 __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
     __shared__ u32 shc[8];
     __shared__ long long shm[8];
     __shared__ u32 ic[256];
     __shared__ long long im[256];
+    // the write pass stages whole cells and lists the survivors by rank, the
+    // count passes stage keys
+    extern __shared__ __align__(16) unsigned char psm[];
+    Cell* const stage = reinterpret_cast<Cell*>(psm);
+    u64* const skey = reinterpret_cast<u64*>(psm);
+    u64* const spos = reinterpret_cast<u64*>(stage + kPlacePad);
+    unsigned short* const sidx = reinterpret_cast<unsigned short*>(spos + kPlaceChunk);
     if (MODE == 1 && a.dirty[blockIdx.x] == 0) return;
     const u64 c = 1ull << a.log2c;
     const u32 hshift = a.B - a.log2c;
-    const u64 i0 = u64(blockIdx.x) * kPlaceChunk + u64(threadIdx.x) * kPlaceItems;
-    u64 ks[kPlaceItems], vs[kPlaceItems];
+    const u64 c0 = u64(blockIdx.x) * kPlaceChunk;
+    const u64 i0 = c0 + u64(threadIdx.x) * kPlaceItems;
+    {
+        u64 k[kPlaceItems], v[kPlaceItems];
 #pragma unroll
-    for (int q = 0; q < kPlaceItems; q += 2) {
-        ks[q] = ks[q + 1] = kEmpty;
-        vs[q] = vs[q + 1] = 0;
-        if (i0 + q + 1 < a.n)
-            ld_pair_nc(a.srt + i0 + q, ks[q], vs[q], ks[q + 1], vs[q + 1]);  // i0 is even: 32-byte aligned
-        else if (i0 + q < a.n)
-            ld_cell_nc(a.srt + i0 + q, ks[q], vs[q]);
+        for (int q = 0; q < kPlaceItems; ++q) {
+            const u64 i = c0 + u32(q) * 256 + threadIdx.x;
+            k[q] = kEmpty;
+            v[q] = 0;
+            if (i < a.n) {
+                if (MODE == 2) ld_cell_nc(a.srt + i, k[q], v[q]);
+                else k[q] = ld_key(a.srt + i);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kPlaceItems; ++q) {
+            const u32 j = padded(u32(q) * 256 + threadIdx.x);
+            if (MODE == 2) {
+                stage[j].key = k[q];
+                stage[j].val = v[q];
+            } else {
+                skey[j] = k[q];
+            }
+        }
     }
+    // the thread's eight flags are one word (flags of a chunk start 8-byte aligned)
+    u64 fl = 0;
+    if (MODE != 0) {
+        if (i0 + kPlaceItems <= a.n) {
+            fl = *reinterpret_cast<const u64*>(a.flags + i0);
+        } else {
+            for (int q = 0; q < kPlaceItems; ++q)
+                if (i0 + q < a.n) fl |= u64(a.flags[i0 + q]) << (8 * q);
+        }
+    }
+    __syncthreads();
+    const u32 s0 = threadIdx.x * (kPlaceItems + 1);  // padded(threadIdx.x * kPlaceItems)
+    u64 ks[kPlaceItems];
+#pragma unroll
+    for (int q = 0; q < kPlaceItems; ++q) ks[q] = MODE == 2 ? stage[s0 + q].key : skey[s0 + q];
+    u64 ss[kPlaceItems];  // sort keys: each hash is computed once
+#pragma unroll
+    for (int q = 0; q < kPlaceItems; ++q) ss[q] = sort_key(ks[q], a.B);
     u32 sv = 0;
     if (MODE == 0) {
-        const u64 knext = i0 + kPlaceItems < a.n ? ld_key(a.srt + i0 + kPlaceItems) : kEmpty;
+        u64 knext = kEmpty;
+        if (i0 + kPlaceItems < a.n)
+            knext = threadIdx.x < 255 ? skey[s0 + kPlaceItems + 1] : ld_key(a.srt + i0 + kPlaceItems);
+        const u64 snext = sort_key(knext, a.B);
 #pragma unroll
         for (int q = 0; q < kPlaceItems; ++q) {
             if (i0 + q >= a.n) continue;
-            const unsigned char f = survivor_first(a, i0 + q, ks[q], q + 1 < kPlaceItems ? ks[q + 1] : knext);
-            a.flags[i0 + q] = f;
+            const unsigned char f =
+                q + 1 < kPlaceItems
+                    ? survivor_first(a, i0 + q, ks[q], ss[q], ks[(q + 1) % kPlaceItems], ss[(q + 1) % kPlaceItems])
+                    : survivor_first(a, i0 + q, ks[q], ss[q], knext, snext);
+            fl |= u64(f) << (8 * q);
             if (f == 1) sv |= 1u << q;
             if (f == 2) a.deferred[atomicAdd(&a.ex->n_deferred, 1u)] = u32(i0 + q);
+        }
+        if (i0 + kPlaceItems <= a.n) {
+            *reinterpret_cast<u64*>(a.flags + i0) = fl;
+        } else {
+            for (int q = 0; q < kPlaceItems; ++q)
+                if (i0 + q < a.n) a.flags[i0 + q] = (unsigned char)(fl >> (8 * q));
         }
     } else {
 #pragma unroll
         for (int q = 0; q < kPlaceItems; ++q)
-            if (i0 + q < a.n && a.flags[i0 + q] == 1) sv |= 1u << q;
+            if (((fl >> (8 * q)) & 255u) == 1u) sv |= 1u << q;
     }
     Agg loc = {0u, kNegInf};
 #pragma unroll
     for (int q = 0; q < kPlaceItems; ++q) {
         if (!((sv >> q) & 1u)) continue;
-        const Agg x = {1u, (long long)(sort_key(ks[q], a.B) >> hshift)};
+        const Agg x = {1u, (long long)(ss[q] >> hshift)};
         loc = agg_join(loc, x);
     }
     Agg tot;
@@ -398,39 +461,64 @@ __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
         const Agg left = {ic[threadIdx.x - 1], im[threadIdx.x - 1]};
         carry = agg_join(carry, left);
     }
-    // the chunk's survivors, by rank, with their positions: staged so that
+    // the chunk's survivors, by rank, with their positions, so that
     // consecutive threads then store consecutive survivors (rising positions)
-    extern __shared__ __align__(16) unsigned char psm[];
-    Cell* const stage = reinterpret_cast<Cell*>(psm);
-    u64* const spos = reinterpret_cast<u64*>(stage + kPlaceChunk);
 #pragma unroll
     for (int q = 0; q < kPlaceItems; ++q) {
         if (!((sv >> q) & 1u)) continue;
-        const u64 home = sort_key(ks[q], a.B) >> hshift;
+        const u64 home = ss[q] >> hshift;
         const u64 rank = carry.c;
         const long long hm = (long long)home - (long long)rank;
         const long long m = carry.m > hm ? carry.m : hm;
         const u32 j = carry.c - first.c;
         spos[j] = rank + u64(m);
-        stage[j].key = ks[q];
-        stage[j].val = vs[q];
+        sidx[j] = (unsigned short)(s0 + q);
         const Agg x = {1u, (long long)home};
         carry = agg_join(carry, x);
     }
     __syncthreads();
     for (u32 j = threadIdx.x; j < tot.c; j += 256) {
         const u64 p = spos[j];
+        if (p < c && a.dense) continue;
+        const Cell cl = stage[sidx[j]];
         if (p < c) {
-            a.cells[p] = stage[j];
+            a.cells[p] = cl;
         } else {
             const u64 rank = u64(first.c) + j;
-            a.ov[rank] = stage[j];
+            a.ov[rank] = cl;
             atomicMin(&a.ex->first_ov, rank);
         }
     }
+    if (!a.dense) return;
+    // dense: the cells from after the last survivor of the chunks before to
+    // this chunk's last one (the last chunk: to the end of the table), a
+    // window of kPlaceWin cells at a time through a map from cell to survivor
+    unsigned short* const map = sidx + kPlaceChunk;
+    const bool last = blockIdx.x + 1 == gridDim.x;
+    u64 w0 = first.c ? u64((long long)first.c + first.m) : 0;
+    u64 end = tot.c ? spos[tot.c - 1] + 1 : w0;
+    if (last || end > c) end = c;
+    const Cell zero = {0ull, 0ull};
+    u32 j = threadIdx.x;  // this thread's next survivor
+    for (; w0 < end; w0 += kPlaceWin) {
+        const u32 len = end - w0 < kPlaceWin ? u32(end - w0) : kPlaceWin;
+        for (u32 x = threadIdx.x; x < kPlaceWin / 4; x += 256) reinterpret_cast<u64*>(map)[x] = ~0ull;
+        __syncthreads();
+        for (; j < tot.c && spos[j] < w0 + len; j += 256) map[spos[j] - w0] = sidx[j];
+        __syncthreads();
+        for (u32 x = threadIdx.x; x < len; x += 256) {
+            const unsigned short i = map[x];
+            a.cells[w0 + x] = i == 0xffffu ? zero : stage[i];
+        }
+        __syncthreads();
+    }
 }
 
-u64 place_smem_bytes() { return size_t(kPlaceChunk) * (sizeof(Cell) + sizeof(u64)); }
+template <int MODE>
+u64 place_smem_bytes() {
+    return MODE == 2 ? size_t(kPlacePad) * sizeof(Cell) + size_t(kPlaceChunk) * (sizeof(u64) + 2) + kPlaceWin * 2
+                     : size_t(kPlacePad) * sizeof(u64);
+}
 
 // ---------------------------------------------------------------------------
 // Deferred survivor tests: one CTA per deferred cell scans the rest of its run
@@ -489,34 +577,65 @@ __global__ void __launch_bounds__(256) build_resolve_kernel(PlaceArgs a) {
     }
 }
 
-// One CTA: exclusive prefixes of the chunk joins, the survivor count S.
+// One CTA: exclusive prefixes of the chunk joins, the survivor count S; kScanJoins
+// joins at a time through shared memory, eight consecutive ones a thread
+// (padded as in the placement), one block scan for each.  (256 joins at a time
+// took 69 us for 2^14 chunks, 8192 at a time by 1024 threads 30 us.)
+constexpr u32 kScanJoins = 2048;
+
 __global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 np, BuildExtra* ex) {
+    __shared__ Agg st[kScanJoins / 8 * 9];
     __shared__ u32 shc[8];
     __shared__ long long shm[8];
-    __shared__ u32 ic[256];
-    __shared__ long long im[256];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     Agg carry = {0u, kNegInf};
-    for (u64 b = 0; b < np; b += 256) {
-        const u64 i = b + threadIdx.x;
-        Agg x = {0u, kNegInf};
-        if (i < np) x = parts[i];
-        Agg tot;
-        const Agg incl = block_incl_agg(x, tot, shc, shm);
-        ic[threadIdx.x] = incl.c;
-        im[threadIdx.x] = incl.m;
-        __syncthreads();
-        if (i < np) {
-            // the join has no inverse (max), so the exclusive prefix is the
-            // carry joined with the previous thread's inclusive one
-            Agg left = {0u, kNegInf};
-            if (threadIdx.x > 0) {
-                left.c = ic[threadIdx.x - 1];
-                left.m = im[threadIdx.x - 1];
-            }
-            parts[i] = agg_join(carry, left);
+    for (u64 b = 0; b < np; b += kScanJoins) {
+#pragma unroll
+        for (u32 q = 0; q < kScanJoins / 256; ++q) {
+            const u32 j = q * 256 + threadIdx.x;
+            st[j + j / 8] = b + j < np ? parts[b + j] : Agg{0u, kNegInf};
         }
         __syncthreads();
-        carry = agg_join(carry, tot);
+        Agg* const mine = st + threadIdx.x * 9;
+        Agg x = mine[0];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) x = agg_join(x, mine[q]);
+        for (int o = 1; o < 32; o <<= 1) {
+            Agg y;
+            y.c = __shfl_up_sync(0xffffffffu, x.c, o);
+            y.m = __shfl_up_sync(0xffffffffu, x.m, o);
+            if (lane >= o) x = agg_join(y, x);
+        }
+        if (lane == 31) {
+            shc[w] = x.c;
+            shm[w] = x.m;
+        }
+        Agg left;
+        left.c = __shfl_up_sync(0xffffffffu, x.c, 1);
+        left.m = __shfl_up_sync(0xffffffffu, x.m, 1);
+        if (lane == 0) left = {0u, kNegInf};
+        __syncthreads();
+        Agg pre = carry;
+        for (int j = 0; j < 8; ++j) {
+            const Agg t = {shc[j], shm[j]};
+            if (j < w) pre = agg_join(pre, t);
+            carry = agg_join(carry, t);
+        }
+        // the join has no inverse (max), so prefixes are carried forward
+        pre = agg_join(pre, left);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const Agg y = mine[q];
+            mine[q] = pre;
+            pre = agg_join(pre, y);
+        }
+        __syncthreads();
+#pragma unroll
+        for (u32 q = 0; q < kScanJoins / 256; ++q) {
+            const u32 j = q * 256 + threadIdx.x;
+            if (b + j < np) parts[b + j] = st[j + j / 8];
+        }
+        __syncthreads();
     }
     if (threadIdx.x == 0) {
         ex->S = carry.c;
@@ -597,6 +716,7 @@ PlaceArgs place_args(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildE
     a.deferred = reinterpret_cast<u32*>(base + L.off_def);
     a.dirty = base + L.off_dirty;
     a.cells = nullptr;
+    a.dense = 0;
     // the survivors past the last cell go to whichever sort buffer does not
     // hold the sorted cells
     Cell* b0 = reinterpret_cast<Cell*>(base);
@@ -655,24 +775,33 @@ cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scrat
     const PlaceArgs a = place_args(sorted, n, log2c, scratch, ex);
     cudaError_t e = cudaMemsetAsync(a.dirty, 0, L.nchunks, s);
     if (e != cudaSuccess) return e;
-    build_place_kernel<0><<<unsigned(L.nchunks), 256, 0, s>>>(a);
+    build_place_kernel<0><<<unsigned(L.nchunks), 256, place_smem_bytes<0>(), s>>>(a);
     // deferred survivor tests (both kernels return at once when there are none)
     build_resolve_kernel<<<unsigned(sm_count() * 4), 256, 0, s>>>(a);
-    build_place_kernel<1><<<unsigned(L.nchunks), 256, 0, s>>>(a);
+    build_place_kernel<1><<<unsigned(L.nchunks), 256, place_smem_bytes<1>(), s>>>(a);
     build_place_scan_kernel<<<1, 256, 0, s>>>(a.parts, L.nchunks, ex);
     for (int i = 0; i < 4; ++i) count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, void* scratch, BuildExtra* ex,
-                               DevState* st, const u64* vals, cudaStream_t s) {
+// New cells are written dense by a batch of at least an eighth of their
+// number: whole sectors, empty cells included, so they need not be zeroed
+// first (a merge of 2^25 + 2^22 pairs into 2^26 cells: 160 us of zeroing and a
+// 313 us write, against one of 310 us).  Below that one chunk's range
+// grows past what a CTA should write.  Cells that are zero already take the
+// survivors alone.
+bool build_place_dense(u64 n, u32 log2c) { return n >= (1ull << log2c) / 8; }
+
+cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, bool dense, void* scratch,
+                               BuildExtra* ex, DevState* st, const u64* vals, cudaStream_t s) {
     const Layout L(n);
     PlaceArgs a = place_args(sorted, n, log2c, scratch, ex);
     a.cells = cells;
+    a.dense = dense ? 1 : 0;
     cudaError_t e = cudaFuncSetAttribute(build_place_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(place_smem_bytes()));
+                                         int(place_smem_bytes<2>()));
     if (e != cudaSuccess) return e;
-    build_place_kernel<2><<<unsigned(L.nchunks), 256, place_smem_bytes(), s>>>(a);
+    build_place_kernel<2><<<unsigned(L.nchunks), 256, place_smem_bytes<2>(), s>>>(a);
     build_finish_kernel<<<1, 32, 0, s>>>(cells, log2c, a.ov, ex, st, vals);
     count_launch();
     count_launch();

@@ -76,7 +76,7 @@ cudaError_t launch_shrink(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log2
 // launch_build_sort sorts the batch's cells by the top build_sort_bits(log2c)
 // hash bits (stable) and routes keys 0 / ~0; launch_build_count counts the
 // survivors (the last copy of each key) into ex->S; launch_build_place writes
-// them into the zeroed cells, wraps the tail and sets I, D and the special
+// them into the cells (zeroed ones unless dense), wraps the tail and sets I, D and the special
 // slots.  n < 2^32.
 struct BuildExtra {
     u64 sp_last[2];  // 1 + input position of the last key 0 / ~0 (0: none)
@@ -92,8 +92,11 @@ cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c
                               const Cell** sorted, BuildExtra** ex, cudaStream_t s);
 cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildExtra* ex,
                                cudaStream_t s);
-cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, void* scratch, BuildExtra* ex,
-                               DevState* st, const u64* vals, cudaStream_t s);
+cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, bool dense, void* scratch,
+                               BuildExtra* ex, DevState* st, const u64* vals, cudaStream_t s);
+// Whether cells that are not zero yet are better written dense (every cell,
+// empty ones too) than zeroed first.
+bool build_place_dense(u64 n, u32 log2c);
 
 // Exclusive scan of m u32 in place (three kernels); `part` holds
 // scan_partials(m) u32.

@@ -1196,7 +1196,8 @@ cht_status cht_build(cht_handle h, const uint64_t* keys, const uint64_t* vals, u
         }
     }
     if (e == cudaSuccess)
-        e = cht::launch_build_place(sorted, n, h->cells, h->log2c, scratch, ex, h->st, static_cast<const u64*>(dv), s);
+        e = cht::launch_build_place(sorted, n, h->cells, h->log2c, false, scratch, ex, h->st, static_cast<const u64*>(dv),
+                                    s);
     lib_free(scratch, sbytes, s);
     if (e != cudaSuccess) return cuda_status(e);
     h->i_bound = n;
@@ -1248,7 +1249,8 @@ cht_status cht_merge(cht_handle h, const uint64_t* keys, const uint64_t* vals, u
     cudaError_t e = cht::launch_compact_live(h->cells, h->log2c, ck, cv, cmp, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ck + live, dk, n * 8, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(cv + live, dv, n * 8, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(cells, 0, cbytes, s);
+    const bool dense = cht::build_place_dense(tot, nl);
+    if (e == cudaSuccess && !dense) e = cudaMemsetAsync(cells, 0, cbytes, s);
     const Cell* sorted = nullptr;
     cht::BuildExtra* ex = nullptr;
     if (e == cudaSuccess)
@@ -1267,7 +1269,7 @@ cht_status cht_merge(cht_handle h, const uint64_t* keys, const uint64_t* vals, u
         }
     }
     // the finish kernel sets I = survivors, D = 0 and the special slots the batch names
-    if (e == cudaSuccess) e = cht::launch_build_place(sorted, tot, cells, nl, bld, ex, h->st, cv, s);
+    if (e == cudaSuccess) e = cht::launch_build_place(sorted, tot, cells, nl, dense, bld, ex, h->st, cv, s);
     lib_free(scratch, sbytes, s);
     if (e != cudaSuccess) {
         lib_free(cells, cbytes, s);
