@@ -7,12 +7,12 @@
 //
 // GB300 mapping.
 //   1. LSD radix sort of the (key, value) cells by the top B bits of the hash
-//      (B = 32 for tables of up to 2^32 cells), 8 bits per pass: a histogram
-//      kernel (one CTA per tile of 2048 cells), an exclusive scan of the
-//      digit-major histogram, and a stable scatter (warp ranks from ballots
-//      of the digit bits, warp offsets in shared memory).  The first pass reads
-//      the caller's key and value arrays and notes keys 0 / ~0 (for the special
-//      slots or the reserved status bit, both set only once the build is sure).
+//      (B = 32 for tables of up to 2^32 cells), 8 bits per pass: one kernel
+//      counts the digits of all passes, then each pass reads and writes the
+//      cells once, tiles of 4096 cells finding their places by decoupled
+//      look-back.  The first pass reads the caller's key and value arrays; the
+//      count notes keys 0 / ~0 (for the special slots or the reserved status
+//      bit, both set only once the build is sure).
 //   2. Placement as a scan: with r_i the number of survivors before i,
 //      P_i = r_i + max over survivors j <= i of (home_j - r_j), so a scan of
 //      (count, max) pairs under (C1, M1) + (C2, M2) = (C1 + C2,
@@ -29,8 +29,9 @@ namespace cht {
 namespace {
 
 constexpr int kSortThreads = 256;
+constexpr int kPassThreads = 512;
 constexpr int kSortItems = 8;
-constexpr u32 kSortTile = kSortThreads * kSortItems;  // cells per radix tile
+constexpr u32 kSortTile = kPassThreads * kSortItems;  // cells per radix tile
 constexpr int kScanThreads = 256;
 constexpr u32 kScanChunk = kScanThreads * 16;          // u32 per scan chunk
 constexpr int kPlaceItems = 8;
@@ -78,70 +79,129 @@ __device__ __forceinline__ u32 block_incl_u32(u32 x, u32& total, u32* sh) {
 // ---------------------------------------------------------------------------
 // radix sort
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(SortSrc src, u64 n, u32 B, u32 shift, u32* hist,
-                                                                  u64 ntiles, BuildExtra* ex, int full_keys) {
-    __shared__ u32 bins[256];
-    bins[threadIdx.x] = 0;
+constexpr int kDigits = 256;
+constexpr int kMaxPasses = 5;  // sort keys of at most 40 bits
+
+// The digit counts of every pass in one read of the keys (8 bytes a pair,
+// where a count before each pass read the whole cells again).  Also notes keys
+// 0 / ~0: they take the special slots (the last copy's value) or set the
+// reserved status bit; they never enter the table.
+__global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const u64* keys, u64 n, u32 B, u32* hist,
+                                                                   BuildExtra* ex, int full_keys) {
+    __shared__ u32 bins[kMaxPasses][kDigits];
+    const int passes = int(B / 8);
+    for (int p = 0; p < passes; ++p) bins[p][threadIdx.x] = 0;
     __syncthreads();
-    const u64 base = u64(blockIdx.x) * kSortTile;
-    for (int q = 0; q < kSortItems; ++q) {
-        const u64 i = base + u64(q) * kSortThreads + threadIdx.x;
-        if (i >= n) break;
-        u64 k, v;
-        load_src(src, i, k, v);
-        atomicAdd(&bins[u32(sort_key(k, B) >> shift) & 255u], 1u);
-        if (!src.cells && is_reserved(k)) {
-            // first pass: keys 0 / ~0 take the special slots (the last copy's
-            // value) or set the reserved status bit; they never enter the table
-            if (full_keys)
-                atomicMax(&ex->sp_last[k == kEmpty ? 0 : 1], i + 1);
-            else
-                atomicOr(&ex->reserved, 1ull);
+    const u64 step = u64(gridDim.x) * (kSortThreads * 8);
+    for (u64 base = u64(blockIdx.x) * (kSortThreads * 8); base < n; base += step) {
+        u64 k[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const u64 i = base + u32(q) * kSortThreads + threadIdx.x;
+            k[q] = i < n ? keys[i] : 1;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const u64 i = base + u32(q) * kSortThreads + threadIdx.x;
+            if (i >= n) break;
+            const u64 s = sort_key(k[q], B);
+            for (int p = 0; p < passes; ++p) atomicAdd(&bins[p][u32(s >> (8 * p)) & 255u], 1u);
+            if (is_reserved(k[q])) {
+                if (full_keys)
+                    atomicMax(&ex->sp_last[k[q] == kEmpty ? 0 : 1], i + 1);
+                else
+                    atomicOr(&ex->reserved, 1ull);
+            }
         }
     }
     __syncthreads();
-    hist[u64(threadIdx.x) * ntiles + blockIdx.x] = bins[threadIdx.x];
+    for (int p = 0; p < passes; ++p)
+        if (bins[p][threadIdx.x]) atomicAdd(&hist[p * kDigits + threadIdx.x], bins[p][threadIdx.x]);
 }
 
-// Stable scatter of one tile: warp w ranks its 256 cells (8 steps of 32
-// consecutive ones): eight ballots give each lane the lanes with its digit,
-// a per-warp counter in shared memory the count of earlier steps.  The warps'
-// per-digit counts and the tile's digit counts are then scanned, the tile is
-// reordered by digit in shared memory (stable), and written out from there:
-// consecutive threads write consecutive cells of a digit's run, so the
-// stores coalesce.
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(SortSrc src, Cell* dst, u64 n, u32 B,
-                                                                     u32 shift, const u32* offs, u64 ntiles) {
-    constexpr int kW = kSortThreads / 32;
+// A tile's digit counts on their way to prefixes: bits 0-31 the count (of this
+// tile, or of all tiles up to it), bits 32-33 which (kTileCount, kTilePrefix),
+// from bit 34 the pass + 1, so that one zeroed array serves all passes.
+constexpr u64 kTileCount = 1ull << 32, kTilePrefix = 2ull << 32;
+constexpr u32 kMaxPolls = 1u << 22;  // a few seconds
+
+struct PassArgs {
+    SortSrc src;
+    Cell* dst;
+    u64 n;
+    u32 B, pass;
+    const u32* hist;  // this pass's digit counts
+    u64* tiles;       // [tile][kDigits]
+    u32* ticket;      // this pass's tile counter (zero before the launch)
+};
+
+// Digit `d` in the tiles before `tile`, counted from the cells themselves:
+// what a lookback falls back on if a tile's counts never appear.
+__device__ __noinline__ u32 recount_digit(const PassArgs& a, u32 tile, u32 d) {
+    u32 sum = 0;
+    for (u64 i = 0; i < u64(tile) * kSortTile; ++i) {
+        u64 k, v;
+        load_src(a.src, i, k, v);
+        sum += (u32(sort_key(k, a.B) >> (8 * a.pass)) & 255u) == d;
+    }
+    return sum;
+}
+
+// One stable 8-bit pass.  A tile ranks its cells (warp w has 256 of them, 8
+// steps of 32 consecutive ones: eight ballots give each lane the lanes with
+// its digit, a per-warp counter in shared memory the count of earlier steps),
+// publishes its digit counts, and gets the counts of the tiles before it by
+// looking back over theirs (decoupled look-back, Merrill & Garland, "Single-pass
+// Parallel Prefix Scan with Decoupled Look-back", 2016; used for radix sorting by
+// Adinets & Merrill, "Onesweep", arXiv 2206.01784): one read and one write of
+// the cells per pass and no count or scan kernels between.  Tiles come from a
+// ticket, so those looked back at are running or done.  The tile is reordered
+// by digit in shared memory (stable) and written from there: consecutive
+// threads write consecutive cells of a digit's run, so the stores coalesce.
+// Bound by shared memory (random 16-byte stores of the reordering).  2^25
+// pairs, a pass: count + scan + scatter 390 us -> 330 us; 2048 to 8192 cells a
+// tile and looking back at 1 to 24 tiles at a time are slower.
+template <bool kFirst>
+__global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(PassArgs a) {
+    constexpr int kW = kPassThreads / 32;
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
-    Cell* const stage = reinterpret_cast<Cell*>(smem);                        // kSortTile cells
-    u32(*const wcnt)[257] = reinterpret_cast<u32(*)[257]>(stage + kSortTile);  // [kW][257]
-    u32* const goff = &wcnt[kW][0];                                          // 256
-    u32* const tstart = goff + 256;                                          // 256
-    unsigned char* const sdig = reinterpret_cast<unsigned char*>(tstart + 256);  // kSortTile
+    Cell* const stage = reinterpret_cast<Cell*>(smem);                             // kSortTile cells
+    unsigned short(*const wcnt)[kDigits + 2] = reinterpret_cast<unsigned short(*)[kDigits + 2]>(stage + kSortTile);
+    u32* const goff = reinterpret_cast<u32*>(&wcnt[kW][0]);                        // place of a digit's run - its slot
+    unsigned char* const sdig = reinterpret_cast<unsigned char*>(goff + kDigits);  // kSortTile
+    __shared__ u32 sh[2][8];
+    __shared__ u32 s_tile;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const u32 below = (1u << lane) - 1u;
-    for (int j = threadIdx.x; j < kW * 257; j += kSortThreads) (&wcnt[0][0])[j] = 0;
-    goff[threadIdx.x] = offs[u64(threadIdx.x) * ntiles + blockIdx.x];
+    const u32 shift = 8 * a.pass;
+    if (threadIdx.x == 0) s_tile = atomicAdd(a.ticket, 1u);
+    for (u32 j = threadIdx.x; j < u32(kW) * (kDigits + 2) / 2; j += kPassThreads) reinterpret_cast<u32*>(wcnt)[j] = 0;
     __syncthreads();
-
-    const u64 tbase = u64(blockIdx.x) * kSortTile;
+    const u32 tile = s_tile;
+    const u64 tbase = u64(tile) * kSortTile;
     const u64 base = tbase + u64(w) * (32 * kSortItems);
     u64 ks[kSortItems], vs[kSortItems];
-    u32 dg[kSortItems], rk[kSortItems];
+    u32 dr[kSortItems];  // digit << 16 | rank in the warp
     // all loads first (in flight together), then the ranking votes
 #pragma unroll
     for (int q = 0; q < kSortItems; ++q) {
         const u64 i = base + u64(q) * 32 + lane;
         ks[q] = 0;
         vs[q] = 0;
-        if (i < n) load_src(src, i, ks[q], vs[q]);
+        if (i < a.n) {
+            if (kFirst) {
+                ks[q] = a.src.keys[i];
+                vs[q] = a.src.vals[i];
+            } else {
+                ld_cell_nc(a.src.cells + i, ks[q], vs[q]);
+            }
+        }
     }
 #pragma unroll
     for (int q = 0; q < kSortItems; ++q) {
-        const u64 i = base + u64(q) * 32 + lane;
-        const bool valid = i < n;
-        const u32 d = valid ? u32(sort_key(ks[q], B) >> shift) & 255u : 0u;
+        const bool valid = base + u64(q) * 32 + lane < a.n;
+        const u32 d = u32(sort_key(ks[q], a.B) >> shift) & 255u;
         // lanes with the same digit: eight ballots, one per digit bit
         u32 peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
@@ -149,48 +209,102 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(SortSrc src
             const u32 m = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
             peers &= ((d >> bit) & 1u) ? m : ~m;
         }
-        dg[q] = valid ? d : 256u;  // past the end: a bin never stored
-        const u32 b = wcnt[w][dg[q]];
-        rk[q] = b + __popc(peers & below);
+        const u32 b = wcnt[w][d];
+        dr[q] = (d << 16) | (b + __popc(peers & below));
         __syncwarp();
-        if (valid && (peers & below) == 0u) wcnt[w][d] = b + __popc(peers);  // the group's lowest lane
+        if (valid && (peers & below) == 0u) wcnt[w][d] = (unsigned short)(b + __popc(peers));  // the lowest lane
         __syncwarp();
     }
     __syncthreads();
-    {   // per digit: exclusive scan over the warps, then over the digits
-        const int d = threadIdx.x;
-        u32 run = 0;
+    if (threadIdx.x < kDigits) {
+        // the tile's count of this thread's digit (and exclusive over the warps)
+        const u32 d = threadIdx.x;
+        u32 cnt = 0;
+#pragma unroll
         for (int x = 0; x < kW; ++x) {
             const u32 t = wcnt[x][d];
-            wcnt[x][d] = run;
-            run += t;
+            wcnt[x][d] = (unsigned short)cnt;
+            cnt += t;
         }
-        u32 tot;
-        const u32 incl = block_incl_u32(run, tot, tstart);  // uses tstart[0..7] as scratch
-        tstart[d] = incl - run;
+        const u64 tag = u64(a.pass + 1) << 34;
+        volatile u64* const mine = a.tiles + u64(tile) * kDigits + d;
+        *mine = tag | (tile == 0 ? kTilePrefix : kTileCount) | cnt;
+        // where the digit's run starts, in the tile and in the output
+        const u32 h = a.hist[d];
+        u32 x = cnt, g = h;
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 y = __shfl_up_sync(0xffffffffu, x, o), z = __shfl_up_sync(0xffffffffu, g, o);
+            if (lane >= o) {
+                x += y;
+                g += z;
+            }
+        }
+        if (lane == 31) {
+            sh[0][w] = x;
+            sh[1][w] = g;
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // the eight warps with a digit per thread
+        u32 slot = x - cnt, place = g - h;
+        for (int j = 0; j < w; ++j) {
+            slot += sh[0][j];
+            place += sh[1][j];
+        }
+#pragma unroll
+        for (int y = 0; y < kW; ++y) wcnt[y][d] = (unsigned short)(wcnt[y][d] + slot);
+        u32 before = 0;
+        if (tile > 0) {
+            u32 polls = 0;
+            for (u32 t = tile;;) {
+                u64 v[4];  // four tiles at a time, the loads in flight together
+#pragma unroll
+                for (u32 u = 0; u < 4; ++u)
+                    v[u] = u < t ? *(volatile u64*)(a.tiles + u64(t - 1 - u) * kDigits + d) : 0;
+                bool done = false, wait = false;
+                u32 used = 0;
+#pragma unroll
+                for (u32 u = 0; u < 4; ++u) {
+                    if (done || wait) continue;
+                    if ((v[u] >> 34) != a.pass + 1) {
+                        wait = true;
+                        continue;
+                    }
+                    before += u32(v[u]);
+                    ++used;
+                    done = (v[u] & kTilePrefix) != 0;
+                }
+                if (done) break;
+                t -= used;
+                if (wait && ++polls > kMaxPolls) {
+                    before = recount_digit(a, tile, d);
+                    break;
+                }
+            }
+            *mine = tag | kTilePrefix | (before + cnt);
+        }
+        goff[d] = place + before - slot;
     }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kSortItems; ++q) {
-        if (dg[q] < 256u) {
-            const u32 j = tstart[dg[q]] + wcnt[w][dg[q]] + rk[q];
+        if (base + u64(q) * 32 + lane < a.n) {
+            const u32 d = dr[q] >> 16, j = wcnt[w][d] + (dr[q] & 0xffffu);
             Cell cl;
             cl.key = ks[q];
             cl.val = vs[q];
             stage[j] = cl;
-            sdig[j] = (unsigned char)dg[q];
+            sdig[j] = (unsigned char)d;
         }
     }
     __syncthreads();
-    const u32 cnt = n - tbase < kSortTile ? u32(n - tbase) : kSortTile;
-    for (u32 j = threadIdx.x; j < cnt; j += kSortThreads) {
-        const u32 d = sdig[j];
-        dst[u64(goff[d]) + (j - tstart[d])] = stage[j];
+    const u32 cnt = a.n - tbase < kSortTile ? u32(a.n - tbase) : kSortTile;
+    for (u32 j = threadIdx.x; j < cnt; j += kPassThreads) {
+        const u32 to = goff[sdig[j]] + j;
+        if (to < a.n) a.dst[to] = stage[j];
     }
 }
 
-u64 scatter_smem_bytes() {
-    return size_t(kSortTile) * sizeof(Cell) + size_t(kSortThreads / 32) * 257 * 4 + 512 * 4 + kSortTile;
+constexpr size_t pass_smem_bytes() {
+    return size_t(kSortTile) * sizeof(Cell) + size_t(kPassThreads / 32) * (kDigits + 2) * 2 + kDigits * 4 + kSortTile;
 }
 
 // ---------------------------------------------------------------------------
@@ -679,27 +793,25 @@ __global__ void build_finish_kernel(Cell* cells, u32 log2c, const Cell* ov, Buil
 u32 build_sort_bits(u32 log2c) { return log2c <= 32 ? 32u : 8u * ((log2c + 7u) / 8u); }
 
 namespace {
-// Scratch layout: two sort buffers, the digit histogram and its scan
-// partials, the chunk joins, the survivor flags, the deferred list, the
+// Scratch layout: two sort buffers, the tiles' digit prefixes, the chunk joins, the survivor flags, the deferred list, the
 // chunks' recount marks, the counters.
+constexpr u64 kCountBytes = (kMaxPasses * (kDigits + 1) * 4 + 255) & ~255ull;
 struct Layout {
-    u64 ntiles, hist_n, nparts, nchunks;
-    u64 off_buf1, off_hist, off_part, off_parts, off_flags, off_def, off_dirty, off_ex, total;
+    u64 ntiles, nchunks;
+    u64 off_buf1, off_tiles, off_parts, off_flags, off_def, off_dirty, off_ex, off_counts, total;
     explicit Layout(u64 n) {
         auto al = [](u64 x) { return (x + 255) & ~255ull; };
         ntiles = (n + kSortTile - 1) / kSortTile;
-        hist_n = 256 * ntiles;
-        nparts = (hist_n + kScanChunk - 1) / kScanChunk;
         nchunks = (n + kPlaceChunk - 1) / kPlaceChunk;
         off_buf1 = al(n * sizeof(Cell));
-        off_hist = off_buf1 + al(n * sizeof(Cell));
-        off_part = off_hist + al(hist_n * 4);
-        off_parts = off_part + al(nparts * 4);
+        off_tiles = off_buf1 + al(n * sizeof(Cell));
+        off_parts = off_tiles + al(ntiles * kDigits * sizeof(u64));
         off_flags = off_parts + al(nchunks * sizeof(Agg));
         off_def = off_flags + al(n);
         off_dirty = off_def + al(n * 4);
         off_ex = off_dirty + al(nchunks);
-        total = off_ex + al(sizeof(BuildExtra));
+        off_counts = off_ex + al(sizeof(BuildExtra));  // digit counts and tile tickets of the passes
+        total = off_counts + kCountBytes;
     }
 };
 
@@ -737,34 +849,52 @@ cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c
     const Layout L(n);
     unsigned char* base = static_cast<unsigned char*>(scratch);
     Cell* buf[2] = {reinterpret_cast<Cell*>(base), reinterpret_cast<Cell*>(base + L.off_buf1)};
-    u32* hist = reinterpret_cast<u32*>(base + L.off_hist);
-    u32* part = reinterpret_cast<u32*>(base + L.off_part);
     BuildExtra* ex = reinterpret_cast<BuildExtra*>(base + L.off_ex);
-    cudaError_t e = cudaMemsetAsync(ex, 0, sizeof(BuildExtra), s);
+    u32* counts = reinterpret_cast<u32*>(base + L.off_counts);
+    u64* tiles = reinterpret_cast<u64*>(base + L.off_tiles);
+    cudaError_t e = cudaMemsetAsync(ex, 0, L.total - L.off_ex, s);  // ex, the counts and the tickets
+    if (e == cudaSuccess) e = cudaMemsetAsync(tiles, 0, L.ntiles * kDigits * sizeof(u64), s);
     if (e != cudaSuccess) return e;
-    SortSrc src;
-    src.cells = nullptr;
-    src.keys = keys;
-    src.vals = vals;
-    e = cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(scatter_smem_bytes()));
-    if (e != cudaSuccess) return e;
+    u64 cgrid = u64(sm_count()) * 8;
+    if (cgrid > (n + kSortThreads * 8 - 1) / (kSortThreads * 8)) cgrid = (n + kSortThreads * 8 - 1) / (kSortThreads * 8);
+    radix_count_kernel<<<unsigned(cgrid), kSortThreads, 0, s>>>(keys, n, B, counts, ex, full_keys);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    constexpr size_t smem = pass_smem_bytes();
+    for (auto fn : {radix_pass_kernel<true>, radix_pass_kernel<false>}) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+    }
+    PassArgs a;
+    a.src.cells = nullptr;
+    a.src.keys = keys;
+    a.src.vals = vals;
+    a.n = n;
+    a.B = B;
+    a.tiles = tiles;
     int cur = 0;
-    for (u32 shift = 0; shift < B; shift += 8) {
-        radix_hist_kernel<<<unsigned(L.ntiles), kSortThreads, 0, s>>>(src, n, B, shift, hist, L.ntiles, ex,
-                                                                    full_keys);
+    for (a.pass = 0; a.pass < B / 8; ++a.pass) {
+        a.dst = buf[cur];
+        a.hist = counts + a.pass * kDigits;
+        a.ticket = counts + kMaxPasses * kDigits + a.pass;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(unsigned(L.ntiles));
+        cfg.blockDim = dim3(kPassThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];  // the next pass's launch overlaps this one's tail
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, a.pass == 0 ? radix_pass_kernel<true> : radix_pass_kernel<false>, a);
         count_launch();
-        e = scan_exclusive(hist, L.hist_n, part, s);
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        radix_scatter_kernel<<<unsigned(L.ntiles), kSortThreads, scatter_smem_bytes(), s>>>(src, buf[cur], n, B,
-                                                                                          shift, hist, L.ntiles);
-        count_launch();
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        src.cells = buf[cur];
+        a.src.cells = buf[cur];
         cur ^= 1;
     }
-    *sorted = src.cells;
+    *sorted = a.src.cells;
     *ex_out = ex;
     return cudaSuccess;
 }
