@@ -838,6 +838,112 @@ PlaceArgs place_args(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildE
 }
 }  // namespace
 
+namespace {
+// ---------------------------------------------------------------------------
+// Merge of two runs sorted by sort key (a table's live cells and a batch), the
+// first run's cells before the second's where sort keys are equal: the stable
+// sort of their concatenation, in one pass.  Merge path (Green, McColl & Bader,
+// "GPU Merge Path", 2012): a binary search over the cells finds where each
+// tile of kPlaceChunk output cells begins in both runs (a kernel of its own,
+// one thread per tile: ~25 dependent reads, which took 5/8 of the time when
+// each tile's CTA waited for its own); the tile's two parts go to shared memory
+// and each thread merges kPlaceItems cells of it.
+// ---------------------------------------------------------------------------
+struct MergeArgs {
+    const Cell* x;  // nx cells
+    const Cell* y;  // ny cells
+    u64 nx, ny;
+    u32 B;
+    u32* split;  // per tile: cells of x before it
+    Cell* out;
+};
+
+// How many of the first `diag` merged cells come from x.
+__device__ __forceinline__ u64 merge_split(const MergeArgs& a, u64 diag) {
+    u64 lo = diag > a.ny ? diag - a.ny : 0, hi = diag < a.nx ? diag : a.nx;
+    while (lo < hi) {
+        const u64 mid = (lo + hi) / 2;
+        if (sort_key(ld_key(a.x + mid), a.B) <= sort_key(ld_key(a.y + (diag - 1 - mid)), a.B)) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+__global__ void __launch_bounds__(128) merge_split_kernel(MergeArgs a) {
+    const u64 tot = a.nx + a.ny, t = u64(blockIdx.x) * 128 + threadIdx.x, d = t * kPlaceChunk;
+    if (d < tot + kPlaceChunk) a.split[t] = u32(merge_split(a, d < tot ? d : tot));
+}
+
+__global__ void __launch_bounds__(256) merge_runs_kernel(MergeArgs a) {
+    extern __shared__ __align__(16) unsigned char msm[];
+    Cell* const stage = reinterpret_cast<Cell*>(msm);            // x's part, then y's
+    u64* const sk = reinterpret_cast<u64*>(stage + kPlaceChunk);  // their sort keys
+    unsigned short* const from = reinterpret_cast<unsigned short*>(sk + kPlaceChunk);
+    const u64 tot = a.nx + a.ny;
+    const u64 d0 = u64(blockIdx.x) * kPlaceChunk, d1 = d0 + kPlaceChunk < tot ? d0 + kPlaceChunk : tot;
+    const u64 x0 = a.split[blockIdx.x], y0 = d0 - x0;
+    const u32 nx = u32(a.split[blockIdx.x + 1] - x0), m = u32(d1 - d0), ny = m - nx;
+#pragma unroll
+    for (int q = 0; q < kPlaceItems; ++q) {
+        const u32 j = u32(q) * 256 + threadIdx.x;
+        if (j < m) {
+            Cell cl;
+            ld_cell_nc(j < nx ? a.x + x0 + j : a.y + y0 + (j - nx), cl.key, cl.val);
+            stage[j] = cl;
+            sk[j] = sort_key(cl.key, a.B);
+        }
+    }
+    __syncthreads();
+    // this thread's cells of the tile: split, then a serial merge
+    const u32 g0 = threadIdx.x * kPlaceItems < m ? threadIdx.x * kPlaceItems : m;
+    u32 lo = g0 > ny ? g0 - ny : 0, hi = g0 < nx ? g0 : nx;
+    while (lo < hi) {
+        const u32 mid = (lo + hi) / 2;
+        if (sk[mid] <= sk[nx + g0 - 1 - mid]) lo = mid + 1;
+        else hi = mid;
+    }
+    u32 i = lo, j = g0 - lo;
+#pragma unroll
+    for (int q = 0; q < kPlaceItems; ++q) {
+        if (g0 + q < m) {
+            const bool take_x = j >= ny || (i < nx && sk[i] <= sk[nx + j]);
+            from[g0 + q] = (unsigned short)(take_x ? i : nx + j);
+            if (take_x) ++i;
+            else ++j;
+        }
+    }
+    __syncthreads();
+    for (u32 t = threadIdx.x; t < m; t += 256) a.out[d0 + t] = stage[from[t]];
+}
+}  // namespace
+
+cudaError_t launch_build_merge(const Cell* x, u64 nx, const Cell* y, u64 ny, u32 log2c, void* scratch,
+                               const Cell** merged, cudaStream_t s) {
+    MergeArgs a;
+    a.x = x;
+    a.y = y;
+    a.nx = nx;
+    a.ny = ny;
+    a.B = build_sort_bits(log2c);
+    a.out = static_cast<Cell*>(scratch);
+    constexpr size_t smem = size_t(kPlaceChunk) * (sizeof(Cell) + sizeof(u64) + 2);
+    const cudaError_t e = cudaFuncSetAttribute(merge_runs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    const u64 tot = nx + ny, tiles = (tot + kPlaceChunk - 1) / kPlaceChunk;
+    // (the sort's tile prefixes are not used by a merge: 2 KB per 4096 cells)
+    a.split = reinterpret_cast<u32*>(static_cast<unsigned char*>(scratch) + Layout(tot).off_tiles);
+    merge_split_kernel<<<unsigned((tiles + 1 + 127) / 128), 128, 0, s>>>(a);
+    merge_runs_kernel<<<unsigned(tiles), 256, smem, s>>>(a);
+    count_launch();
+    count_launch();
+    *merged = a.out;
+    return cudaGetLastError();
+}
+
+Cell* build_spare_cells(void* scratch, u64 n) {
+    return reinterpret_cast<Cell*>(static_cast<unsigned char*>(scratch) + Layout(n).off_buf1);
+}
+
 u64 build_scratch_bytes(u64 n) { return Layout(n).total; }
 
 u64 scan_partials(u64 m) { return (m + kScanChunk - 1) / kScanChunk; }

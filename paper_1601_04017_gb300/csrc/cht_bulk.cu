@@ -232,16 +232,59 @@ constexpr u32 kCompactPerWarp = kCompactChunk / kPWarps;  // 512 cells, 16 windo
 
 __device__ __forceinline__ bool live_key(u64 k) { return k != kEmpty && k != kTomb; }
 
-__global__ void __launch_bounds__(kPThreads) live_count_kernel(const Cell* cells, u64 c, u32* counts) {
+constexpr int kMaxTombWalk = 32;  // tombstones a live cell looks back over
+
+// Counts, and the check of the order.  Live cells across an empty cell are in
+// order already (a cell's home lies behind the last empty cell before it), so
+// each live cell compares its sort key with the live cell before it in its
+// cluster, and its home with its index (a cluster that wraps past the last
+// cell holds high hashes at low indexes).  Tables made by a bulk build or
+// merge are in order as long as nothing else has put cells in; those filled
+// one by one hardly ever are.
+template <bool kCheck>
+__global__ void __launch_bounds__(kPThreads) live_count_kernel(const Cell* cells, u32 log2c, u32 B, u32* counts,
+                                                               u32* unsorted) {
     __shared__ u32 wsum[kPWarps];
+    const u64 c = 1ull << log2c;
     const u64 base = u64(blockIdx.x) * kCompactChunk;
+    const int lane = threadIdx.x & 31;
     u32 cnt = 0;
-    for (u32 j = threadIdx.x; j < kCompactChunk; j += kPThreads) {
-        const u64 i = base + j;
-        if (i < c && live_key(cells[i].key)) ++cnt;
+    bool bad = false;
+    constexpr int U = 8;
+    static_assert(kCompactChunk % (kPThreads * U) == 0, "whole steps");
+    for (u32 j0 = 0; j0 < kCompactChunk; j0 += kPThreads * U) {
+        u64 k[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u64 i = base + j0 + u * kPThreads + threadIdx.x;
+            k[u] = i < c ? cells[i].key : kEmpty;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const u64 i = base + j0 + u * kPThreads + threadIdx.x;
+            const bool live = live_key(k[u]);
+            if (live) ++cnt;
+            if (!kCheck) continue;
+            const u64 h = fmix64(k[u]);
+            // the cell before: the lane before's, or (lane 0, tombstones) from memory
+            u64 pk = __shfl_up_sync(0xffffffffu, k[u], 1), ph = __shfl_up_sync(0xffffffffu, h, 1);
+            if (live) {
+                if (lane == 0 || pk == kTomb) {
+                    u64 p = i;
+                    int left = kMaxTombWalk;
+                    do {
+                        pk = p > 0 ? cells[--p].key : kEmpty;
+                    } while (pk == kTomb && --left > 0);
+                    bad |= pk == kTomb;  // not looked at: not known to be in order
+                    ph = fmix64(pk);
+                }
+                bad |= (pk != kEmpty && (ph >> (64u - B)) > (h >> (64u - B))) || (h >> (64u - log2c)) > i;
+            }
+        }
     }
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = cnt;
+    if (kCheck && __any_sync(0xffffffffu, bad) && lane == 0) *unsorted = 1;
+    if (lane == 0) wsum[threadIdx.x >> 5] = cnt;
     __syncthreads();
     if (threadIdx.x == 0) {
         u32 t = 0;
@@ -250,31 +293,44 @@ __global__ void __launch_bounds__(kPThreads) live_count_kernel(const Cell* cells
     }
 }
 
+// A warp keeps its 16 windows' cells in registers between counting and writing
+// them: the table is read once.
 __global__ void __launch_bounds__(kPThreads) live_write_kernel(const Cell* cells, u64 c, const u32* offs,
-                                                               u64* keys_out, u64* vals_out) {
+                                                               u64* keys_out, u64* vals_out, Cell* cells_out) {
     __shared__ u32 wcount[kPWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const u32 below = (1u << lane) - 1u;
     const u64 base = u64(blockIdx.x) * kCompactChunk + u64(w) * kCompactPerWarp;
-    u32 cnt = 0;
-    for (u32 j = 0; j < kCompactPerWarp; j += 32) {
-        const u64 i = base + j + lane;
-        cnt += __popc(__ballot_sync(0xffffffffu, i < c && live_key(cells[i].key)));
+    constexpr int U = int(kCompactPerWarp / 32);
+    u64 k[U], v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const u64 i = base + u * 32 + lane;
+        k[u] = kEmpty;
+        v[u] = 0;
+        if (i < c) ld_cell_nc(cells + i, k[u], v[u]);
     }
+    u32 cnt = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) cnt += __popc(__ballot_sync(0xffffffffu, live_key(k[u])));
     if (lane == 0) wcount[w] = cnt;
     __syncthreads();
     u64 out = offs[blockIdx.x];
     for (int x = 0; x < w; ++x) out += wcount[x];
-    for (u32 j = 0; j < kCompactPerWarp; j += 32) {
-        const u64 i = base + j + lane;
-        u64 k = 0, v = 0;
-        if (i < c) ld_cell_nc(cells + i, k, v);
-        const bool lv = i < c && live_key(k);
-        const u32 m = __ballot_sync(0xffffffffu, lv);
-        if (lv) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const u32 m = __ballot_sync(0xffffffffu, live_key(k[u]));
+        if (live_key(k[u])) {
             const u64 o = out + __popc(m & below);
-            keys_out[o] = k;
-            vals_out[o] = v;
+            if (cells_out) {
+                Cell cl;
+                cl.key = k[u];
+                cl.val = v[u];
+                cells_out[o] = cl;
+            } else {
+                keys_out[o] = k[u];
+                vals_out[o] = v[u];
+            }
         }
         out += __popc(m);
     }
@@ -412,23 +468,44 @@ cudaError_t launch_sorted16(const OpArgs& a, void* scratch, PartitionRun run, vo
     return cudaSuccess;
 }
 
-u64 compact_scratch_bytes(u32 log2c) {
-    const u64 nchunks = ((1ull << log2c) + kCompactChunk - 1) / kCompactChunk;
-    return align256((nchunks + 1) * 4) + align256(scan_partials(nchunks + 1) * 4);
+namespace {
+struct CompactScratch {
+    u64 nchunks, o_part, o_flag, total;
+    explicit CompactScratch(u32 log2c) {
+        nchunks = ((1ull << log2c) + kCompactChunk - 1) / kCompactChunk;
+        o_part = align256((nchunks + 1) * 4);
+        o_flag = o_part + align256(scan_partials(nchunks + 1) * 4);
+        total = o_flag + 256;
+    }
+};
+}  // namespace
+
+u64 compact_scratch_bytes(u32 log2c) { return CompactScratch(log2c).total; }
+
+cudaError_t launch_compact_count(const Cell* cells, u32 log2c, bool check, void* scratch, u32** unsorted,
+                                 cudaStream_t s) {
+    const CompactScratch L(log2c);
+    unsigned char* b = static_cast<unsigned char*>(scratch);
+    u32* counts = reinterpret_cast<u32*>(b);
+    *unsorted = reinterpret_cast<u32*>(b + L.o_flag);
+    cudaError_t e = cudaMemsetAsync(*unsorted, 0, sizeof(u32), s);
+    if (e != cudaSuccess) return e;
+    if (check)
+        live_count_kernel<true><<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, log2c, build_sort_bits(log2c), counts,
+                                                                        *unsorted);
+    else
+        live_count_kernel<false><<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, log2c, build_sort_bits(log2c), counts,
+                                                                         *unsorted);
+    count_launch();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return scan_exclusive_u32(counts, L.nchunks, reinterpret_cast<u32*>(b + L.o_part), s);
 }
 
-cudaError_t launch_compact_live(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, void* scratch,
-                                cudaStream_t s) {
-    const u64 c = 1ull << log2c;
-    const u64 nchunks = (c + kCompactChunk - 1) / kCompactChunk;
-    u32* counts = static_cast<u32*>(scratch);
-    u32* part = reinterpret_cast<u32*>(static_cast<unsigned char*>(scratch) + align256((nchunks + 1) * 4));
-    live_count_kernel<<<unsigned(nchunks), kPThreads, 0, s>>>(cells, c, counts);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if ((e = scan_exclusive_u32(counts, nchunks, part, s)) != cudaSuccess) return e;
-    live_write_kernel<<<unsigned(nchunks), kPThreads, 0, s>>>(cells, c, counts, keys_out, vals_out);
+cudaError_t launch_compact_write(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, Cell* cells_out,
+                                 void* scratch, cudaStream_t s) {
+    const CompactScratch L(log2c);
+    live_write_kernel<<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, 1ull << log2c, static_cast<const u32*>(scratch),
+                                                               keys_out, vals_out, cells_out);
     count_launch();
     return cudaGetLastError();
 }

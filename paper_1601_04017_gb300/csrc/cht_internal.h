@@ -98,6 +98,13 @@ cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c
 // empty ones too) than zeroed first.
 bool build_place_dense(u64 n, u32 log2c);
 
+// Merge of two runs that are sorted as launch_build_sort sorts (x before y on
+// equal sort keys) into the first buffer of a scratch block for nx + ny cells;
+// build_spare_cells is its second one, which may hold the runs.
+cudaError_t launch_build_merge(const Cell* x, u64 nx, const Cell* y, u64 ny, u32 log2c, void* scratch,
+                               const Cell** merged, cudaStream_t s);
+Cell* build_spare_cells(void* scratch, u64 n);
+
 // Exclusive scan of m u32 in place (three kernels); `part` holds
 // scan_partials(m) u32.
 u64 scan_partials(u64 m);
@@ -131,12 +138,17 @@ cudaError_t launch_partitioned(const OpArgs& a, PartitionIO io, void* scratch, P
 u64 sorted16_scratch_bytes(u64 n, bool codes);
 cudaError_t launch_sorted16(const OpArgs& a, void* scratch, PartitionRun run, void* ctx, cudaStream_t s);
 
-// The live cells (neither empty nor tombstone) in cell index order into
-// keys_out / vals_out (deterministic; the bulk merge's table side).  Scratch:
-// compact_scratch_bytes(log2c).
+// The live cells (neither empty nor tombstone) in cell index order
+// (deterministic; the bulk merge's table side), in two steps over one scratch
+// block of compact_scratch_bytes(log2c): launch_compact_count counts them and,
+// with check, notes in *unsorted (a word of the scratch) whether that order is
+// not the one launch_build_sort would give them; launch_compact_write writes them as two
+// arrays (keys_out, vals_out) or, with keys_out null, as cells.
 u64 compact_scratch_bytes(u32 log2c);
-cudaError_t launch_compact_live(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, void* scratch,
-                                cudaStream_t s);
+cudaError_t launch_compact_count(const Cell* cells, u32 log2c, bool check, void* scratch, u32** unsorted,
+                                 cudaStream_t s);
+cudaError_t launch_compact_write(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, Cell* cells_out,
+                                 void* scratch, cudaStream_t s);
 
 // In-kernel growth (cht_grow.cu, Sec. 4.3.2): one cooperative launch runs an
 // insert / insertOrUpdate batch on a growable table, migrating between
