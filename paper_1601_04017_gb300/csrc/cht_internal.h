@@ -233,6 +233,7 @@ struct EngineArgs {
     unsigned max_backoff_ns;   // longest sleep between two polls of a dependency counter
     int any_reuse;             // some table of the launch reuses tombstones
     int any_full;              // some table of the launch has the full key space
+    int chained;               // a table's chain of levels outlasts the launch's work (plan_order)
     // optional snapshot at the end of the launch: the last warp to finish
     // writes I, D of tables[snap_tables[i]] to snap_out[2i], snap_out[2i + 1]
     // (n_snap = 0: none); warps_done: a counter, zero before the launch
@@ -263,10 +264,11 @@ namespace cht {
 // Consecutive levels of one table that are one item each are grouped: the
 // first is a queue item that leads the rest.  chunk_ops: operations per
 // item (32..256, a power of two), 0 = sized per table from the length of
-// its chain of levels.  Returns the number of queue items; `chunks` holds
-// them followed by the followers.
+// its chain of levels.  *chained: some table's chain is estimated to outlast
+// the work of the whole plan.  Returns the number of queue items; `chunks`
+// holds them followed by the followers.
 u64 plan_order(const std::vector<EngineBatch>& batches, size_t n_tables, int chunk_ops,
-               std::vector<EngineChunk>& chunks);
+               std::vector<EngineChunk>& chunks, bool* chained);
 
 // Runtime services for translation units outside the runtime.
 struct TableInfo {

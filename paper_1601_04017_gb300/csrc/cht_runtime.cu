@@ -683,8 +683,9 @@ constexpr u32 kMaxGroup = 4096;
 }  // namespace
 
 u64 plan_order(const std::vector<EngineBatch>& batches, size_t n_tables, int chunk_ops,
-               std::vector<EngineChunk>& chunks) {
+               std::vector<EngineChunk>& chunks, bool* chained) {
     const size_t nb = batches.size();
+    *chained = false;
     constexpr u32 kNone = ~0u;
     // Dependency levels.  A find right after a find of the same table does
     // not wait for it (finds do not modify the table, so both see the state
@@ -739,6 +740,7 @@ u64 plan_order(const std::vector<EngineBatch>& batches, size_t n_tables, int chu
             }
         for (size_t t = 0; t < n_tables; ++t) {
             int j = 0;
+            if (chain[4 * t] > work_us) *chained = true;
             while (j < 3 && chain[4 * t + j] > work_us) ++j;
             chunk_of[t] = kChunkOps >> j;
         }
@@ -1616,6 +1618,7 @@ struct cht_plan {
     unsigned long long* d_counters = nullptr;  // [0] queue cursor, [1 + t] table t's done items
     u32* d_status = nullptr;
     u64 n_batches = 0, n_chunks = 0;
+    bool chained = false;
     u64 bytes_tables = 0, bytes_batches = 0, bytes_chunks = 0, bytes_counters = 0;
     std::vector<cht::EngineBatch> batches;  // host copy: work items are rebuilt when chunk_ops changes
     cht_plan_config cfg{0, 0, 0, 0, 0, 0, 0, 0};
@@ -1653,6 +1656,7 @@ cht::EngineArgs plan_args(const cht_plan* p) {
     e.max_backoff_ns = p->cfg.poll_ns > 0 ? unsigned(p->cfg.poll_ns) : 8192u;
     e.any_reuse = 0;
     e.any_full = 0;
+    e.chained = p->chained;
     for (const cht_table* h : p->tables) {
         e.any_reuse |= h->cfg.reuse_tombstones;
         e.any_full |= h->cfg.full_key_space;
@@ -1755,7 +1759,7 @@ cht_status cht_plan_create(const cht_batch_op* ops, uint64_t n_ops, cht_plan_han
     }
     // work items, round by round; need = the table's items in earlier levels
     std::vector<cht::EngineChunk> chunks;
-    const u64 n_queue = cht::plan_order(batches, p->tables.size(), 0, chunks);
+    const u64 n_queue = cht::plan_order(batches, p->tables.size(), 0, chunks, &p->chained);
     std::vector<cht::EngineTable> tabs(p->tables.size());
     for (size_t t = 0; t < p->tables.size(); ++t) {
         tabs[t].cells = p->tables[t]->cells;
@@ -1806,7 +1810,8 @@ cht_status cht_plan_set_config(cht_plan_handle p, const cht_plan_config* cfg) {
         return CHT_ERR_INVALID_ARG;
     if (c.chunk_ops != p->cfg.chunk_ops && p->n_chunks > 0) {  // rebuild the work items
         std::vector<cht::EngineChunk> chunks;
-        const u64 n_queue = cht::plan_order(p->batches, p->tables.size(), c.chunk_ops, chunks);
+        bool chained = false;
+        const u64 n_queue = cht::plan_order(p->batches, p->tables.size(), c.chunk_ops, chunks, &chained);
         DeviceGuard g(p->device);
         cht::EngineChunk* d = nullptr;
         u64 bytes = 0;
@@ -1820,6 +1825,7 @@ cht_status cht_plan_set_config(cht_plan_handle p, const cht_plan_config* cfg) {
         p->d_chunks = d;
         p->bytes_chunks = bytes;
         p->n_chunks = n_queue;
+        p->chained = chained;
     }
     p->cfg = c;
     return CHT_OK;

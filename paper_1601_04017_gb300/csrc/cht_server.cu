@@ -383,9 +383,10 @@ cht_status admit_and_launch(cht_server* s, u32* admitted) {
     // work items sized per table from its chain of dependent requests; if
     // that needs more metadata than a step may use, take 64-operation items
     std::vector<cht::EngineChunk> chunks;
-    u64 n_queue = cht::plan_order(batches, nt, 0, chunks);
+    bool chained = false, recut = false;
+    u64 n_queue = cht::plan_order(batches, nt, 0, chunks, &chained);
     if (chunks.size() > s->max_step_items) {
-        n_queue = cht::plan_order(batches, nt, 64, chunks);
+        n_queue = cht::plan_order(batches, nt, 64, chunks, &recut);  // (the chains are what they were)
         st.rec.recut = 1;
     }
     std::vector<u32> touched;
@@ -446,6 +447,7 @@ cht_status admit_and_launch(cht_server* s, u32* admitted) {
     e.max_backoff_ns = 8192;
     e.any_reuse = 0;
     e.any_full = 0;
+    e.chained = chained;
     for (const cht::EngineTable& et : tabs) {
         e.any_reuse |= int(et.flags & cht::kTabReuse);
         e.any_full |= int((et.flags & cht::kTabFullKeys) != 0);
