@@ -46,6 +46,9 @@ struct OpArgs {
 cudaError_t launch_op(Mode mode, const OpArgs& a, int group_width, int lane_cells, int ctas_per_sm,
                       cudaStream_t s);
 
+// Zero cells and zero state.
+cudaError_t launch_clear(Cell* cells, u32 log2c, DevState* st, cudaStream_t s);
+
 // insertOrUpdate (mode kIouAdd or kIouOverwrite) with CTA-level
 // aggregation of equal keys in shared memory before the table is touched.
 // warp_dedup: first combine equal keys of each warp step (extreme skew).

@@ -900,8 +900,8 @@ cht_status cht_create(uint64_t capacity, int growable, cht_stream_t stream, cht_
         delete h;
         return r;
     }
-    if (cudaMemsetAsync(h->cells, 0, h->cap() * sizeof(Cell), s) != cudaSuccess ||
-        cudaMemsetAsync(h->st, 0, sizeof(DevState), s) != cudaSuccess) {
+    if (cht::launch_clear(h->cells, h->log2c, h->st, s) != cudaSuccess) {
+        cudaGetLastError();
         lib_free(h->cells, h->cells_bytes, s);
         lib_free(h->st, sizeof(DevState), s);
         delete h;
@@ -1468,8 +1468,8 @@ cht_status cht_clear(cht_handle h, cht_stream_t stream) {
     DeviceGuard g(h->device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     h->last = s;
-    if (cudaMemsetAsync(h->cells, 0, h->cap() * sizeof(Cell), s) != cudaSuccess) return CHT_ERR_CUDA;
-    if (cudaMemsetAsync(h->st, 0, sizeof(DevState), s) != cudaSuccess) return CHT_ERR_CUDA;
+    const cht_status r = cuda_status(cht::launch_clear(h->cells, h->log2c, h->st, s));
+    if (r != CHT_OK) return r;
     h->i_bound = 0;
     h->i_exact = true;
     return CHT_OK;
