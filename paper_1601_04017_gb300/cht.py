@@ -183,12 +183,28 @@ def _ptr(x, elem_size: int, n: int | None = None, what: str = "array"):
     return ptr, cnt, cuda
 
 
-def _stream(stream, device=None):
-    if stream is not None:
-        return ctypes.c_void_p(int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream))
+_current_raw = None  # () -> handle of torch's current CUDA stream
+
+
+def _find_current_raw():
+    """torch's current stream as a plain handle: asked for on every call, and
+    building a Stream object for it takes 3 us, a third of a small call."""
+    global _current_raw
     import torch
 
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    torch.cuda.current_stream()  # initializes CUDA
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _current_raw = lambda: raw(dev())  # noqa: E731
+    else:
+        _current_raw = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    return _current_raw
+
+
+def _stream(stream):
+    if stream is not None:
+        return ctypes.c_void_p(int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream))
+    return ctypes.c_void_p((_current_raw or _find_current_raw())())
 
 
 def memory_in_use() -> int:

@@ -1026,9 +1026,10 @@ cht_status piece_launch(cht_table* h, cht::Mode mode, const u64* keys, const u64
 cht_status pipelined(cht_table* h, cht::Mode mode, const u64* keys, const u64* vals, u64* vout,
                      unsigned char* codes, u64 n, cudaStream_t s, PieceFn fn, bool* handled) {
     *handled = false;
+    if (n <= kPipeChunk || h->device < 0 || h->device >= 64) return CHT_OK;
     const bool hk = is_host_pointer(keys), hv = vals && is_host_pointer(vals);
     const bool ho = vout && is_host_pointer(vout), hc = codes && is_host_pointer(codes);
-    if (n <= kPipeChunk || !(hk || hv || ho || hc) || h->device < 0 || h->device >= 64) return CHT_OK;
+    if (!(hk || hv || ho || hc)) return CHT_OK;
     DevPipe& P = g_pipe[h->device];
     std::lock_guard<std::mutex> lk(P.mu);
     if (!pipe_ready(h->device)) return CHT_OK;
