@@ -90,14 +90,17 @@ void lib_free(void* p, u64 bytes, cudaStream_t s) {
     g_mem_in_use.fetch_sub(bytes);
 }
 
-bool is_host_pointer(const void* p) {
+// 0: memory of the device, 1: pinned host memory, 2: pageable host memory.
+int host_kind(const void* p) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return true;
+        return 2;
     }
-    return at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeUnregistered;
+    return at.type == cudaMemoryTypeHost ? 1 : at.type == cudaMemoryTypeUnregistered ? 2 : 0;
 }
+
+bool is_host_pointer(const void* p) { return host_kind(p) != 0; }
 
 // Stages host arrays of one call through device buffers on the stream.
 class Staging {
@@ -937,19 +940,35 @@ cht_status cht_get_config(cht_handle h, cht_config* cfg) {
 }
 
 // ---------------------------------------------------------------------------
-// Pipelined staging of host arrays.  A call with host arrays larger than one
-// piece is cut into pieces of kPipeChunk operations that cycle through
-// kPipeSlots device slots: piece i+1 is copied in on a copy stream while piece
-// i runs on the caller's stream and piece i-1's results are copied out on a
-// second copy stream.  Pieces of one batch run one after another on the
-// caller's stream, which is one linearization of the batch (phase semantics
-// hold per piece and across them).  Device arrays are used in place.  The
-// slots (about 420 MB per slot) are allocated on a device's first pipelined
-// call and kept until the process exits; calls on one device take the slots
-// one after another (a host lock around the enqueueing, events on the GPU).
+// Pipelined staging of host arrays.  A call with host arrays runs in pieces:
+// piece i+1 is copied in on a copy stream while piece i runs on the caller's
+// stream and piece i-1's results are copied out on a second copy stream, so
+// the link carries both directions at once and the kernels hide behind it.
+// Pieces of one batch run one after another on the caller's stream, which is
+// one linearization of the batch (phase semantics hold per piece and across
+// them).  Device arrays are used in place.  An eighth of the batch is a piece:
+// fewer leave the first copy in and the last copy out alone on the link, more
+// cost launches (2^24 + 2^22 finds with pinned arrays: pieces of 2^24 1990 us,
+// of an eighth 1361 us; 2^22 staged whole
+// 479 us, in pieces 354 us).  Batches of more than kPipeChunk operations cycle
+// through kPipeSlots device slots (about 420 MB per slot, allocated on a
+// device's first such call and kept until the process exits; pieces of at most
+// kPipeChunk); calls on one device take the slots one after another (a host
+// lock around the enqueueing, events on the GPU).  Batches of kPipeMin to
+// kPipeChunk operations are staged whole, as smaller ones are, and only copied
+// and run in pieces.
 // ---------------------------------------------------------------------------
 constexpr u64 kPipeChunk = 1ull << 24;
+constexpr u64 kPipeMin = 1ull << 20;
+constexpr int kPipePieces = 8;
 constexpr int kPipeSlots = 3;
+
+// operations of a piece of an n-operation batch
+u64 pipe_piece(u64 n) {
+    const u64 unit = 1ull << 16;
+    const u64 p = (n / kPipePieces + unit - 1) / unit * unit;
+    return p < kPipeChunk ? p : kPipeChunk;
+}
 
 struct PipeSlot {
     u64* keys = nullptr;
@@ -963,25 +982,37 @@ struct PipeSlot {
 
 struct DevPipe {
     std::mutex mu;
-    bool tried = false, ok = false;
+    bool tried = false, ok = false;            // the slots
+    bool streams_tried = false, streams = false;  // what every pipelined call needs
     cudaStream_t cin = nullptr, cout = nullptr;
     cudaEvent_t start = nullptr;  // the work on the caller's stream before a call
+    cudaEvent_t in[kPipePieces] = {}, run[kPipePieces] = {}, out = nullptr;  // of a batch staged whole
     PipeSlot slot[kPipeSlots];
     int next = 0;
 };
 DevPipe g_pipe[64];
+
+bool pipe_streams(DevPipe& P) {
+    if (P.streams_tried) return P.streams;
+    P.streams_tried = true;
+    bool ok = cudaStreamCreateWithFlags(&P.cin, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&P.cout, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&P.out, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 0; i < kPipePieces && ok; ++i)
+        ok = cudaEventCreateWithFlags(&P.in[i], cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&P.run[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    P.streams = ok;
+    return ok;
+}
 
 bool pipe_ready(int dev) {
     DevPipe& P = g_pipe[dev];
     if (P.tried) return P.ok;
     P.tried = true;
     const u64 per = kPipeChunk * (8 + 8 + 8 + 1);
-    if (cudaStreamCreateWithFlags(&P.cin, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&P.cout, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    if (!pipe_streams(P)) return false;
     unsigned char* mem = nullptr;
     if (cudaMalloc(&mem, per * kPipeSlots) != cudaSuccess) {
         cudaGetLastError();
@@ -1020,27 +1051,103 @@ cht_status piece_launch(cht_table* h, cht::Mode mode, const u64* keys, const u64
     return launch(h, mode, keys, vals, vout, codes, m, s);
 }
 
+// A batch of kPipeMin .. kPipeChunk operations: device copies of the whole host
+// arrays (as the plain way makes them), copied and run in pieces.
+cht_status pipelined_whole(cht_table* h, cht::Mode mode, const u64* keys, const u64* vals, u64* vout,
+                           unsigned char* codes, u64 n, bool hk, bool hv, bool ho, bool hc, cudaStream_t s, PieceFn fn) {
+    DevPipe& P = g_pipe[h->device];
+    u64 *bk = nullptr, *bv = nullptr, *bo = nullptr;
+    unsigned char* bc = nullptr;
+    cht_status r = CHT_OK;
+    if (hk) r = lib_alloc(reinterpret_cast<void**>(&bk), n * 8, s);
+    if (r == CHT_OK && hv) r = lib_alloc(reinterpret_cast<void**>(&bv), n * 8, s);
+    if (r == CHT_OK && ho) r = lib_alloc(reinterpret_cast<void**>(&bo), n * 8, s);
+    if (r == CHT_OK && hc) r = lib_alloc(reinterpret_cast<void**>(&bc), n, s);
+    auto ok = [&](cudaError_t e) {
+        if (e == cudaSuccess || r != CHT_OK) return;
+        cudaGetLastError();
+        r = CHT_ERR_CUDA;
+    };
+    // the copies in wait for the work already on s (it may write the inputs)
+    if (r == CHT_OK) ok(cudaEventRecord(P.start, s));
+    if (r == CHT_OK) ok(cudaStreamWaitEvent(P.cin, P.start, 0));
+    const u64 piece = pipe_piece(n);
+    bool out = false;
+    u64 lo = 0;
+    for (int i = 0; lo < n && r == CHT_OK; ++i, lo += piece) {
+        const u64 m = n - lo < piece ? n - lo : piece;
+        if (hk) ok(cudaMemcpyAsync(bk + lo, keys + lo, m * 8, cudaMemcpyHostToDevice, P.cin));
+        if (hv) ok(cudaMemcpyAsync(bv + lo, vals + lo, m * 8, cudaMemcpyHostToDevice, P.cin));
+        ok(cudaEventRecord(P.in[i], P.cin));
+        ok(cudaStreamWaitEvent(s, P.in[i], 0));
+        if (r != CHT_OK) break;
+        r = fn(h, mode, hk ? bk + lo : keys + lo, vals ? (hv ? bv + lo : vals + lo) : nullptr,
+               vout ? (ho ? bo + lo : vout + lo) : nullptr, codes ? (hc ? bc + lo : codes + lo) : nullptr, m, s);
+        if (!(ho || hc)) continue;
+        out = true;
+        ok(cudaEventRecord(P.run[i], s));
+        ok(cudaStreamWaitEvent(P.cout, P.run[i], 0));
+        if (ho) ok(cudaMemcpyAsync(vout + lo, bo + lo, m * 8, cudaMemcpyDeviceToHost, P.cout));
+        if (hc) ok(cudaMemcpyAsync(codes + lo, bc + lo, m, cudaMemcpyDeviceToHost, P.cout));
+    }
+    // the call completes on s, and its buffers are freed, once both copy
+    // streams are done with them
+    cudaError_t e = cudaSuccess;
+    if (lo > 0 || r != CHT_OK) {
+        e = cudaEventRecord(P.start, P.cin);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, P.start, 0);
+    }
+    if (out && e == cudaSuccess) {
+        e = cudaEventRecord(P.out, P.cout);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, P.out, 0);
+    }
+    ok(e);
+    lib_free(bk, n * 8, s);
+    lib_free(bv, n * 8, s);
+    lib_free(bo, n * 8, s);
+    lib_free(bc, n, s);
+    return r;
+}
+
 // Runs the call through the pipeline if some array is in host memory and the
-// batch is larger than one piece; *handled = false otherwise (the caller
-// then stages the plain way).
+// batch is large enough; *handled = false otherwise (the caller then stages
+// the plain way).
 cht_status pipelined(cht_table* h, cht::Mode mode, const u64* keys, const u64* vals, u64* vout,
                      unsigned char* codes, u64 n, cudaStream_t s, PieceFn fn, bool* handled) {
     *handled = false;
-    if (n <= kPipeChunk || h->device < 0 || h->device >= 64) return CHT_OK;
-    const bool hk = is_host_pointer(keys), hv = vals && is_host_pointer(vals);
-    const bool ho = vout && is_host_pointer(vout), hc = codes && is_host_pointer(codes);
+    if (n < kPipeMin || h->device < 0 || h->device >= 64) return CHT_OK;
+    const int kinds[4] = {host_kind(keys), vals ? host_kind(vals) : 0, vout ? host_kind(vout) : 0,
+                          codes ? host_kind(codes) : 0};
+    const bool hk = kinds[0] != 0, hv = kinds[1] != 0, ho = kinds[2] != 0, hc = kinds[3] != 0;
+    // (copies of pageable memory hold the host up one after the other: smaller
+    // pieces of them only cost launches)
+    const bool pageable = std::find(kinds, kinds + 4, 2) != kinds + 4;
     if (!(hk || hv || ho || hc)) return CHT_OK;
     DevPipe& P = g_pipe[h->device];
+    if (n <= kPipeChunk) {
+        if (pageable) return CHT_OK;
+        // (a capture keeps the plain way: the copy streams are shared)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return CHT_OK;
+        }
+        std::lock_guard<std::mutex> lk(P.mu);
+        if (!pipe_streams(P)) return CHT_OK;
+        *handled = true;
+        return pipelined_whole(h, mode, keys, vals, vout, codes, n, hk, hv, ho, hc, s, fn);
+    }
     std::lock_guard<std::mutex> lk(P.mu);
     if (!pipe_ready(h->device)) return CHT_OK;
     *handled = true;
+    const u64 piece = pageable ? kPipeChunk : pipe_piece(n);
     // the copies in wait for the work already on s (it may write the inputs)
     if (cudaEventRecord(P.start, s) != cudaSuccess || cudaStreamWaitEvent(P.cin, P.start, 0) != cudaSuccess)
         return CHT_ERR_CUDA;
     bool used[kPipeSlots] = {};
     cht_status r = CHT_OK;
-    for (u64 lo = 0; lo < n && r == CHT_OK; lo += kPipeChunk) {
-        const u64 m = n - lo < kPipeChunk ? n - lo : kPipeChunk;
+    for (u64 lo = 0; lo < n && r == CHT_OK; lo += piece) {
+        const u64 m = n - lo < piece ? n - lo : piece;
         PipeSlot& q = P.slot[P.next];
         used[P.next] = true;
         P.next = (P.next + 1) % kPipeSlots;
