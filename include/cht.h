@@ -103,10 +103,9 @@ typedef enum {
  * 512 below load 0.6, else 1024).  alpha: growth threshold in (0, 1) (Sec. 4.3.2; default 0.5).
  * iou_aggregate: 1 (default) folds equal keys of each window of 1024
  * insertOrUpdate or update operations in shared memory first (one table
- * operation per distinct key and window), and for insertOrUpdate also combines
- * equal keys within each warp step in a window that follows a window with
- * fewer distinct keys than a fifth of its operations; 2 always combines them
- * (insertOrUpdate); 3 first sorts an insertOrUpdate batch by the top 16 bits
+ * operation per distinct key and window); 2 the same (it once also combined
+ * equal keys within each warp step, which the folding now does as fast);
+ * 3 first sorts an insertOrUpdate batch by the top 16 bits
  * of the hash (two stable 8-bit passes, Sec. 4.5 integer sorting) so that the
  * windows -- 4096 operations per 1024-thread CTA -- hold every operation of
  * the keys they see, and puts the result codes back into the caller's order

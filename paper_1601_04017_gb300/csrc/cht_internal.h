@@ -51,12 +51,11 @@ cudaError_t launch_clear(Cell* cells, u32 log2c, DevState* st, cudaStream_t s);
 
 // insertOrUpdate (mode kIouAdd or kIouOverwrite) with CTA-level
 // aggregation of equal keys in shared memory before the table is touched.
-// warp_dedup: first combine equal keys of each warp step (extreme skew).
-cudaError_t launch_iou_aggregated(Mode mode, const OpArgs& a, bool warp_dedup, int ctas_per_sm, cudaStream_t s);
+cudaError_t launch_iou_aggregated(Mode mode, const OpArgs& a, int ctas_per_sm, cudaStream_t s);
 // The same with 1024-thread CTAs and windows of 4096 operations (8192
 // shared-memory slots): for batches sorted by hash, where a window holds the
 // whole groups of a key's operations.  insertOrUpdate modes only.
-cudaError_t launch_iou_aggregated_wide(Mode mode, const OpArgs& a, bool warp_dedup, cudaStream_t s);
+cudaError_t launch_iou_aggregated_wide(Mode mode, const OpArgs& a, cudaStream_t s);
 
 // Cluster-wise migration of `src` (2^src_log2 cells) into `dst`
 // (2^dst_log2 cells, dst_log2 >= src_log2).  dst needs no initialisation:

@@ -157,21 +157,21 @@ cudaError_t launch_mode(const OpArgs& a, int g, int v, int ctas_per_sm, cudaStre
     }
 }
 
-template <int MODE, int WD, bool RE, int BLOCK = kAggBlock>
+template <int MODE, bool RE, int BLOCK = kAggBlock>
 cudaError_t launch_agg(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     constexpr size_t smem = agg_smem_bytes<MODE, BLOCK>();
     static std::atomic<int> occ{0};
     int per_sm = occ.load(std::memory_order_relaxed);
     if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(iou_agg_kernel<MODE, WD, RE, BLOCK>,
+        cudaError_t e = cudaFuncSetAttribute(iou_agg_kernel<MODE, RE, BLOCK>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
         // as much of the unified L1 / shared memory as shared memory as the
         // kernel can use (38 KB per 256-thread CTA, 152 KB per 1024-thread CTA)
-        e = cudaFuncSetAttribute(iou_agg_kernel<MODE, WD, RE, BLOCK>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(iou_agg_kernel<MODE, RE, BLOCK>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  100);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iou_agg_kernel<MODE, WD, RE, BLOCK>, BLOCK, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iou_agg_kernel<MODE, RE, BLOCK>, BLOCK, smem);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
         occ.store(per_sm, std::memory_order_relaxed);
@@ -181,7 +181,7 @@ cudaError_t launch_agg(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     const u64 nwin = (a.n + 4 * BLOCK - 1) / (4 * BLOCK);
     if (grid > nwin) grid = nwin;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_pdl(iou_agg_kernel<MODE, WD, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
+    const cudaError_t e = launch_pdl(iou_agg_kernel<MODE, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -205,45 +205,28 @@ cudaError_t launch_clear(Cell* cells, u32 log2c, DevState* st, cudaStream_t s) {
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_iou_aggregated(Mode mode, const OpArgs& a, bool warp_dedup, int ctas_per_sm, cudaStream_t s) {
+cudaError_t launch_iou_aggregated(Mode mode, const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     const bool re = a.reuse != 0;
-    if (mode == kIouAdd) {
-        if (re)
-            return warp_dedup ? launch_agg<kIouAdd, 2, true>(a, ctas_per_sm, s)
-                              : launch_agg<kIouAdd, 1, true>(a, ctas_per_sm, s);
-        return warp_dedup ? launch_agg<kIouAdd, 2, false>(a, ctas_per_sm, s)
-                          : launch_agg<kIouAdd, 1, false>(a, ctas_per_sm, s);
+    switch (mode) {
+        case kIouAdd: return re ? launch_agg<kIouAdd, true>(a, ctas_per_sm, s) : launch_agg<kIouAdd, false>(a, ctas_per_sm, s);
+        case kIouOverwrite:
+            return re ? launch_agg<kIouOverwrite, true>(a, ctas_per_sm, s)
+                      : launch_agg<kIouOverwrite, false>(a, ctas_per_sm, s);
+        // update: equal keys fold the same way; no cell is filled, so tombstone
+        // reuse does not apply
+        case kUpdAdd: return launch_agg<kUpdAdd, false>(a, ctas_per_sm, s);
+        case kUpdOverwrite: return launch_agg<kUpdOverwrite, false>(a, ctas_per_sm, s);
+        default: return cudaErrorInvalidValue;
     }
-    if (mode == kIouOverwrite) {
-        if (re)
-            return warp_dedup ? launch_agg<kIouOverwrite, 2, true>(a, ctas_per_sm, s)
-                              : launch_agg<kIouOverwrite, 1, true>(a, ctas_per_sm, s);
-        return warp_dedup ? launch_agg<kIouOverwrite, 2, false>(a, ctas_per_sm, s)
-                          : launch_agg<kIouOverwrite, 1, false>(a, ctas_per_sm, s);
-    }
-    // update: equal keys fold the same way; no cell is filled, so neither the
-    // warp pre-reduction nor tombstone reuse applies
-    if (mode == kUpdAdd) return launch_agg<kUpdAdd, 0, false>(a, ctas_per_sm, s);
-    if (mode == kUpdOverwrite) return launch_agg<kUpdOverwrite, 0, false>(a, ctas_per_sm, s);
-    return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_iou_aggregated_wide(Mode mode, const OpArgs& a, bool warp_dedup, cudaStream_t s) {
+cudaError_t launch_iou_aggregated_wide(Mode mode, const OpArgs& a, cudaStream_t s) {
     if (a.n == 0) return cudaSuccess;
     const bool re = a.reuse != 0;
-    if (mode == kIouAdd) {
-        if (re)
-            return warp_dedup ? launch_agg<kIouAdd, 2, true, 1024>(a, 0, s) : launch_agg<kIouAdd, 1, true, 1024>(a, 0, s);
-        return warp_dedup ? launch_agg<kIouAdd, 2, false, 1024>(a, 0, s) : launch_agg<kIouAdd, 1, false, 1024>(a, 0, s);
-    }
-    if (mode == kIouOverwrite) {
-        if (re)
-            return warp_dedup ? launch_agg<kIouOverwrite, 2, true, 1024>(a, 0, s)
-                              : launch_agg<kIouOverwrite, 1, true, 1024>(a, 0, s);
-        return warp_dedup ? launch_agg<kIouOverwrite, 2, false, 1024>(a, 0, s)
-                          : launch_agg<kIouOverwrite, 1, false, 1024>(a, 0, s);
-    }
+    if (mode == kIouAdd) return re ? launch_agg<kIouAdd, true, 1024>(a, 0, s) : launch_agg<kIouAdd, false, 1024>(a, 0, s);
+    if (mode == kIouOverwrite)
+        return re ? launch_agg<kIouOverwrite, true, 1024>(a, 0, s) : launch_agg<kIouOverwrite, false, 1024>(a, 0, s);
     return cudaErrorInvalidValue;
 }
 

@@ -805,12 +805,18 @@ namespace cht {
 // atomicUpdate), whose result -- inserted or updated -- goes to the slot's
 // first operation; every other operation of the key reports "updated"
 // (linearized right after it).  Under skewed keys this turns millions of
-// atomics on one hot cell into one per window.  A warp may first combine the
-// equal keys of its load step with __match_any_sync, which pays off only
-// under extreme skew (many lanes on one shared-memory slot): DEDUP 2 always
-// does, DEDUP 1 (insertOrUpdate's default) does it for a window when the
-// CTA's previous window had fewer distinct keys than a fifth of its
-// operations, DEDUP 0 (update) never.
+// atomics on one hot cell into one per window.
+//
+// What bounds it: with few distinct keys the folding (shared-memory atomics and
+// the instructions around them), with many the flush's random cells.  The
+// sums are two native 32-bit adds (slot_add).  (With 64-bit sums a warp
+// combined its equal keys with match_any first where a window had few distinct
+// ones: 2^26 operations over 2^24 words, s = 0.5 / 1.0 / 1.25 / 1.5: 3.08 / 2.14
+// / 1.59 / 1.20 ms, now 2.87 / 1.95 /
+// 0.96 / 0.61 ms.  Combining in the warp as well costs 0.4 ms at
+// s >= 1.25: the native adds take lanes on one slot at once.  Appending a warp's
+// new slots to the window's list with one add costs 0.2 ms at s = 0.5, and all
+// first looks at the slots ahead of the folding give nothing.)
 // ---------------------------------------------------------------------------
 constexpr int kAggBlock = 256;
 constexpr int kAggWindow = 1024;
@@ -894,6 +900,12 @@ __device__ __forceinline__ unsigned char global_modify(const OpArgs& a, u64 key,
     return kCodeFull;
 }
 
+// A slot for a key: any mixing of its bits will do (keys need not be random).
+__device__ __forceinline__ u32 slot_hash(u64 k) {
+    const u32 x = (u32(k) ^ u32(k >> 32) * 0x85ebca6bu) * 0x9e3779b1u;
+    return x ^ (x >> 15);
+}
+
 // Shared memory of the aggregation kernel: slot keys, values and first ops;
 // for update modes also each operation's slot and each slot's result (every
 // operation on a key reports whether the key was present).
@@ -906,102 +918,113 @@ constexpr size_t agg_smem_bytes() {
            ((MODE == kUpdAdd || MODE == kUpdOverwrite) ? size_t(4 * BLOCK) * 2 + 8 * BLOCK : 0);
 }
 
-// The flush of one window's distinct keys, kAggWindow / kAggBlock at most per
-// thread, with the memory accesses of all of a thread's keys in flight at
-// once: first every key's home sector is loaded, then every key whose sector
-// decides it issues its atomic (the CAS into the empty cell, or the update of
-// its cell), and only the few keys that need more -- a sector without a
-// deciding cell, a CAS lost to another key -- continue one by one with the
-// sector-wise probe from where they stopped.  Same results as probing each key
-// on its own (Algorithm 1 per key; the keys are distinct).
-template <int MODE>
-__device__ __forceinline__ void flush_keys(const OpArgs& a, const u64* fk, const u64* fd, const bool* fv,
-                                           unsigned char* res, u64 cap, u32 shift, u64& n_ins, u64& n_reused,
-                                           u32& sbits) {
-    constexpr int R = kAggWindow / kAggBlock;
+// Sums in a slot are two 32-bit words: shared memory adds 32 bits natively, a
+// 64-bit add is a compare-and-swap loop that lanes on one hot slot repeat for
+// each other.  The carry goes from the low word's old value to the high word,
+// so the sum is exact modulo 2^64.
+__device__ __forceinline__ void slot_add(u32* lo, u32* hi, u32 s, u64 d) {
+    const u32 dl = u32(d);
+    const u32 old = atomicAdd(lo + s, dl);
+    const u32 up = u32(d >> 32) + (old + dl < old ? 1u : 0u);
+    if (up) atomicAdd(hi + s, up);
+}
+
+// The flush of R of a thread's distinct keys of the window, their probe steps
+// issued together: every round loads the next sector of each key still
+// undecided, then issues the atomics of those decided (the CAS into an empty
+// cell, or the update of a cell); a CAS lost to another key goes on with the
+// next cell.  After kFlushRounds the sector-wise probe takes over from where a
+// key stopped.  Same results as probing each key on its own (Algorithm 1 per
+// key; the keys are distinct).  Keys and values stay in their slots fs[r];
+// act: the keys there are.  Two keys at a time (kFlushKeys) keep the kernel at
+// 58 registers and 4 CTAs per SM: 2^26 overwrites at s = 0.5 take 2.99 ms,
+// against 3.21 ms with four first sectors together and their tails one after
+// the other, and 3.73 ms four at a time, which spills.
+constexpr int kFlushRounds = 12;
+constexpr int kFlushKeys = 2;
+
+template <int MODE, int R>
+__device__ __forceinline__ void flush_keys(const OpArgs& a, const u64* skey, const u32* slo, const u32* shi,
+                                           const u32* fs, u32 act, unsigned char* res, u64 cap, u32 shift, u64& n_ins,
+                                           u64& n_reused, u32& sbits) {
     constexpr bool kUpdate = MODE == kUpdAdd || MODE == kUpdOverwrite;
-    const u64 cmask = cap - 1;
-    u64 pos[R], k0[R], v0[R], k1[R], v1[R];
+    Cell* const end = a.cells + cap;
+    Cell* p[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        k0[r] = v0[r] = k1[r] = v1[r] = 0;
-        pos[r] = 0;
-        if (fv[r]) {
-            pos[r] = home_of(fk[r], shift);
-            ld_pair_cg(a.cells + (pos[r] & ~1ull), k0[r], v0[r], k1[r], v1[r]);
-        }
-    }
-    // 0 done, 1 CAS issued, 2 probe on from pos[r]
-    int st[R];
-    Cell old[R];
+    for (int r = 0; r < R; ++r) p[r] = a.cells + ((act >> r) & 1u ? home_of(skey[fs[r]], shift) : 0);
+    for (int round = 0; round < kFlushRounds && act; ++round) {
+        u64 k0[R], v0[R], k1[R], v1[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        st[r] = 0;
-        old[r].key = old[r].val = 0;
-        if (!fv[r]) continue;
-        const u64 key = fk[r];
-        const u64 base = pos[r] & ~1ull;
-        int hit = -1;
-        bool match = false;
-        if ((pos[r] & 1ull) == 0 && (k0[r] == key || k0[r] == kEmpty)) {
-            hit = 0;
-            match = k0[r] == key;
-        } else if (k1[r] == key || k1[r] == kEmpty) {
-            hit = 1;
-            match = k1[r] == key;
-        }
-        if (hit < 0) {
-            st[r] = 2;
-            pos[r] = (base + 2) & cmask;
-            continue;
-        }
-        Cell* cp = a.cells + base + hit;
-        if (match) {
-            if (MODE == kIouAdd || MODE == kUpdAdd) atomicAdd(&cp->val, fd[r]);
-            else atomicExch(&cp->val, fd[r]);
-            res[r] = kUpdate ? kYes : kNo;
-        } else if (kUpdate) {
-            res[r] = kNo;  // an empty cell before the key: absent
-        } else {
-            Cell expect;
-            expect.key = kEmpty;
-            expect.val = 0;
-            Cell desired;
-            desired.key = key;
-            desired.val = fd[r];
-            old[r] = cas_cell(cp, expect, desired);
-            st[r] = 1;
-            pos[r] = base + hit;
-        }
-    }
+        for (int r = 0; r < R; ++r)
+            if ((act >> r) & 1u)
+                ld_pair_cg(reinterpret_cast<const Cell*>(reinterpret_cast<uintptr_t>(p[r]) & ~uintptr_t(31)), k0[r],
+                           v0[r], k1[r], v1[r]);
+        u32 cas = 0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (st[r] != 1) continue;
-        if (old[r].key == kEmpty && old[r].val == 0) {
-            ++n_ins;
-            res[r] = kYes;
-            st[r] = 0;
-        } else if (old[r].key == fk[r]) {  // another copy of the key won the cell: update it
-            Cell* cp = a.cells + pos[r];
-            if (MODE == kIouAdd) atomicAdd(&cp->val, fd[r]);
-            else atomicExch(&cp->val, fd[r]);
-            res[r] = kNo;
-            st[r] = 0;
-        } else {
-            st[r] = 2;
-            pos[r] = (pos[r] + 1) & cmask;
+        for (int r = 0; r < R; ++r) {
+            if (!((act >> r) & 1u)) continue;
+            const u64 key = skey[fs[r]];
+            const bool odd = (reinterpret_cast<uintptr_t>(p[r]) & 16) != 0;
+            const bool h0 = !odd && (k0[r] == key || k0[r] == kEmpty);
+            const u64 k = h0 ? k0[r] : k1[r];
+            Cell* const c = (odd || h0) ? p[r] : p[r] + 1;
+            const u64 d = slo[fs[r]] | u64(shi[fs[r]]) << 32;
+            if (k == key) {
+                if (MODE == kIouAdd || MODE == kUpdAdd) atomicAdd(&c->val, d);
+                else atomicExch(&c->val, d);
+                res[r] = kUpdate ? kYes : kNo;
+                act &= ~(1u << r);
+            } else if (k == kEmpty) {
+                if (kUpdate) {  // an empty cell before the key: absent
+                    res[r] = kNo;
+                    act &= ~(1u << r);
+                } else {
+                    Cell expect, desired;
+                    expect.key = kEmpty;
+                    expect.val = 0;
+                    desired.key = key;
+                    desired.val = d;
+                    const Cell old = cas_cell(c, expect, desired);
+                    k0[r] = old.key;
+                    v0[r] = old.val;
+                    cas |= 1u << r;
+                    p[r] = c;
+                }
+            } else {
+                p[r] = c + 1 == end ? a.cells : c + 1;
+            }
+        }
+        if (!kUpdate) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (!((cas >> r) & 1u)) continue;
+                const u64 key = skey[fs[r]];
+                if (k0[r] == kEmpty && v0[r] == 0) {
+                    ++n_ins;
+                    res[r] = kYes;
+                    act &= ~(1u << r);
+                } else if (k0[r] == key) {  // another copy of the key won the cell: update it
+                    const u64 d = slo[fs[r]] | u64(shi[fs[r]]) << 32;
+                    if (MODE == kIouAdd) atomicAdd(&p[r]->val, d);
+                    else atomicExch(&p[r]->val, d);
+                    res[r] = kNo;
+                    act &= ~(1u << r);
+                } else {
+                    p[r] = p[r] + 1 == end ? a.cells : p[r] + 1;
+                }
+            }
         }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        if (st[r] != 2) continue;
-        const u64 probed = (pos[r] - home_of(fk[r], shift)) & cmask;
-        res[r] = global_modify<MODE, false>(a, fk[r], fd[r], cap, shift, n_ins, n_reused, sbits, pos[r],
-                                            probed == 0 ? cap : probed);
+        if (!((act >> r) & 1u)) continue;
+        const u64 key = skey[fs[r]], pos = u64(p[r] - a.cells), probed = (pos - home_of(key, shift)) & (cap - 1);
+        res[r] = global_modify<MODE, false>(a, key, slo[fs[r]] | u64(shi[fs[r]]) << 32, cap, shift, n_ins, n_reused, sbits,
+                                            pos, probed == 0 ? cap : probed);
     }
 }
 
-template <int MODE, int DEDUP, bool kReuse, int BLOCK = kAggBlock>
+template <int MODE, bool kReuse, int BLOCK = kAggBlock>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) {
     constexpr int kB = BLOCK, kW = 4 * BLOCK, kS = 8 * BLOCK;
     pdl_enter();
@@ -1009,9 +1032,10 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) 
     constexpr bool kAdd = MODE == kIouAdd || MODE == kUpdAdd;
     extern __shared__ __align__(16) unsigned char agg_smem[];
     u64* const skey = reinterpret_cast<u64*>(agg_smem);
-    u64* const sval = skey + kS;
+    u32* const slo = reinterpret_cast<u32*>(skey + kS);  // a slot's value: low and high words (slot_add)
+    u32* const shi = slo + kS;
     // window offset of the slot's first op (< kW: 16 bits)
-    unsigned short* const slead = reinterpret_cast<unsigned short*>(sval + kS);
+    unsigned short* const slead = reinterpret_cast<unsigned short*>(shi + kS);
     unsigned short* const slist = slead + kS;  // the window's claimed slots
     unsigned short* const sslot = slist + kW;                                   // update: op -> slot
     unsigned char* const sres = reinterpret_cast<unsigned char*>(sslot + kW);   // update: slot result
@@ -1021,15 +1045,13 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) 
     u64 n_ins = 0, n_reused = 0;
     u32 sbits = 0;
     __shared__ u32 s_distinct[2];  // distinct keys (claimed slots) of this CTA's window, by window parity
-    __shared__ unsigned long long s_wsum[kB];  // warp pre-reduction: per lane, its group's sum
-    s_wsum[tid] = 0;
     for (int s = tid; s < kS; s += kB) {
         skey[s] = kEmpty;
-        sval[s] = 0;
+        slo[s] = 0;
+        shi[s] = 0;
     }
     if (tid < 2) s_distinct[tid] = 0;
     __syncthreads();
-    bool dedup = DEDUP == 2;
     const u64 nwin = (a.n + kW - 1) / kW;
     // windows: blockIdx.x, + gridDim.x, ... or, with a ticket counter, the
     // next window in batch order (every window already ends in a barrier,
@@ -1057,88 +1079,56 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) 
             wk[j] = idx < a.n ? ld_stream(a.keys + idx) : 0;
             wv[j] = idx < a.n ? ld_stream(a.vals + idx) : 0;
         }
-        // fold the window's operations into the slots
+        // the operations that go on to a slot: not past the end, not reserved
+        u32 valid = 0;
 #pragma unroll
         for (int j = 0; j < kPer; ++j) {
             const u32 off = u32(j * kB + tid);
             const u64 idx = w0 + off;
-            bool valid = idx < a.n;
-            u64 key = 0, d = 0;
+            bool ok = idx < a.n;
             if (kUpdate) sslot[off] = 0xffffu;
-            if (valid) {
-                key = wk[j];
-                d = wv[j];
-                if (is_reserved(key)) {
-                    if (a.full_keys) {
-                        const unsigned char r = special_op<MODE>(a.st, key, d, nullptr);
-                        if (a.codes) a.codes[idx] = r;
-                    } else {
-                        if (a.codes) a.codes[idx] = kCodeReserved;
-                        sbits |= kReserved;
-                    }
-                    valid = false;
+            if (ok && is_reserved(wk[j])) {
+                if (a.full_keys) {
+                    const unsigned char r = special_op<MODE>(a.st, wk[j], wv[j], nullptr);
+                    if (a.codes) a.codes[idx] = r;
+                } else {
+                    if (a.codes) a.codes[idx] = kCodeReserved;
+                    sbits |= kReserved;
                 }
+                ok = false;
             }
-            // optionally, equal keys within the warp first: one lane per key goes
-            // on (dedup is the same for the whole block)
-            const u32 vm = dedup ? __ballot_sync(0xffffffffu, valid) : 0u;
-            if (dedup && valid) {
-                const u32 same = __match_any_sync(vm, key);
-                const int lane = tid & 31;
-                if (kAdd) {
-                    // the group's sum: every lane adds its value into its
-                    // leader's word of a warp-private scratch (a few cycles of
-                    // shared-memory atomics instead of a shuffle round per
-                    // member), the leader takes it and clears the word
-                    const int lead = __ffs(same) - 1;
-                    unsigned long long* const ws = s_wsum + (tid & ~31);
-                    atomicAdd(ws + lead, d);
-                    __syncwarp(vm);
-                    if (lane == lead) {
-                        d = ws[lead];
-                        ws[lead] = 0;
-                    }
-                    __syncwarp(vm);
-                }
-                if (lane != __ffs(same) - 1) {
-                    if (a.codes) a.codes[idx] = kNo;
-                    valid = false;
-                }
-            }
-            if (!valid) continue;
-            u32 s = u32(fmix64(key)) & (kS - 1);
+            if (ok) valid |= 1u << j;
+        }
+        // fold them into the slots
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            if (!((valid >> j) & 1u)) continue;
+            const u64 key = wk[j];
+            u32 s = slot_hash(key) & (kS - 1);
+            bool mine = false;
             for (;;) {
-                const u64 k0 = *reinterpret_cast<volatile u64*>(skey + s);
-                bool mine = false, same = k0 == key;
-                if (k0 == kEmpty) {
-                    const u64 old = atomicCAS(reinterpret_cast<unsigned long long*>(skey + s), kEmpty, key);
-                    mine = old == kEmpty;
-                    same = old == key;
+                u64 k = *reinterpret_cast<volatile u64*>(skey + s);
+                if (k == kEmpty) {
+                    k = atomicCAS(reinterpret_cast<unsigned long long*>(skey + s), kEmpty, key);
+                    mine = k == kEmpty;
                 }
-                if (mine) {
-                    if (kAdd) atomicAdd(reinterpret_cast<unsigned long long*>(sval + s), d);
-                    else sval[s] = d;
-                    slead[s] = (unsigned short)off;
-                    if (kUpdate) sslot[off] = (unsigned short)s;
-                    slist[atomicAdd(&s_distinct[par], 1u)] = (unsigned short)s;
-                    break;
-                }
-                if (same) {
-                    if (kAdd) atomicAdd(reinterpret_cast<unsigned long long*>(sval + s), d);
-                    if (kUpdate) sslot[off] = (unsigned short)s;
-                    else if (a.codes) a.codes[idx] = kNo;
-                    break;
-                }
+                if (mine || k == key) break;
                 s = (s + 1) & (kS - 1);
+            }
+            if (kAdd) {
+                slot_add(slo, shi, s, wv[j]);
+            } else if (mine) {
+                slo[s] = u32(wv[j]);
+                shi[s] = u32(wv[j] >> 32);
+            }
+            if (kUpdate) sslot[j * kB + tid] = (unsigned short)s;
+            else if (a.codes && !mine) a.codes[w0 + u32(j * kB + tid)] = kNo;
+            if (mine) {
+                if (!kUpdate) slead[s] = (unsigned short)(j * kB + tid);
+                slist[atomicAdd(&s_distinct[par], 1u)] = (unsigned short)s;
             }
         }
         __syncthreads();
-        if (DEDUP == 1) {
-            // the next window of this CTA combines within warps if this one had
-            // few distinct keys
-            const u64 ops = a.n - w0 < u64(kW) ? a.n - w0 : u64(kW);
-            dedup = u64(s_distinct[par]) * 2 < ops;
-        }
         if (tid == 0) s_distinct[par ^ 1] = 0;  // the next window's counter (read by all before it)
         // flush: one global operation per distinct key of the window (the
         // dense list of claimed slots; at most kW / kB per thread)
@@ -1147,35 +1137,40 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) 
             for (u32 j = tid; j < nd; j += kB) {
                 const u32 sl = slist[j];
                 const unsigned char r =
-                    global_modify<MODE, kReuse>(a, skey[sl], sval[sl], cap, shift, n_ins, n_reused, sbits);
+                    global_modify<MODE, kReuse>(a, skey[sl], slo[sl] | u64(shi[sl]) << 32, cap, shift, n_ins, n_reused,
+                                                sbits);
                 if (kUpdate) sres[sl] = r;
                 else if (a.codes) a.codes[w0 + slead[sl]] = r;
                 skey[sl] = kEmpty;
-                sval[sl] = 0;
+                slo[sl] = 0;
+                shi[sl] = 0;
             }
         } else {
-            constexpr int R = kW / kB;
-            u64 fk[R], fd[R];
-            bool fv[R];
-            u32 fs[R];
-            unsigned char res[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const u32 j = u32(tid + r * kB);
-                fv[r] = j < nd;
-                fs[r] = fv[r] ? slist[j] : 0u;
-                fk[r] = fv[r] ? skey[fs[r]] : 0;
-                fd[r] = fv[r] ? sval[fs[r]] : 0;
-                res[r] = kNo;
-            }
-            flush_keys<MODE>(a, fk, fd, fv, res, cap, shift, n_ins, n_reused, sbits);
+            for (int h = 0; h < kW / kB; h += kFlushKeys) {
+                u32 fs[kFlushKeys], act = 0;
+                unsigned char res[kFlushKeys];
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (!fv[r]) continue;
-                if (kUpdate) sres[fs[r]] = res[r];
-                else if (a.codes) a.codes[w0 + slead[fs[r]]] = res[r];
-                skey[fs[r]] = kEmpty;
-                sval[fs[r]] = 0;
+                for (int r = 0; r < kFlushKeys; ++r) {
+                    const u32 j = u32(tid + (h + r) * kB);
+                    fs[r] = 0;
+                    res[r] = kNo;
+                    if (j < nd) {
+                        fs[r] = slist[j];
+                        act |= 1u << r;
+                    }
+                }
+                const u32 mine = act;
+                flush_keys<MODE, kFlushKeys>(a, skey, slo, shi, fs, act, res, cap, shift, n_ins, n_reused, sbits);
+#pragma unroll
+                for (int r = 0; r < kFlushKeys; ++r) {
+                    if (!((mine >> r) & 1u)) continue;
+                    if (kUpdate) sres[fs[r]] = res[r];
+                    else if (a.codes) a.codes[w0 + slead[fs[r]]] = res[r];
+                    skey[fs[r]] = kEmpty;
+                    slo[fs[r]] = 0;
+                    shi[fs[r]] = 0;
+                }
             }
         }
         __syncthreads();

@@ -411,7 +411,7 @@ struct KernelCtx {
 cudaError_t run_kernel(const cht::OpArgs& a, void* ctx, cudaStream_t s) {
     const KernelCtx* k = static_cast<const KernelCtx*>(ctx);
     if (aggregated(k->h, k->mode))
-        return cht::launch_iou_aggregated(k->mode, a, k->h->cfg.iou_aggregate == 2, k->h->cfg.ctas_per_sm, s);
+        return cht::launch_iou_aggregated(k->mode, a, k->h->cfg.ctas_per_sm, s);
     const Width w = pick_width(k->h, k->mode, k->n);
     return cht::launch_op(k->mode, a, w.g, w.v, k->h->cfg.ctas_per_sm ? k->h->cfg.ctas_per_sm : w.ctas, s);
 }
@@ -420,7 +420,7 @@ cudaError_t run_kernel(const cht::OpArgs& a, void* ctx, cudaStream_t s) {
 // windows
 cudaError_t run_sorted_agg(const cht::OpArgs& a, void* ctx, cudaStream_t s) {
     const KernelCtx* k = static_cast<const KernelCtx*>(ctx);
-    return cht::launch_iou_aggregated_wide(k->mode, a, false, s);
+    return cht::launch_iou_aggregated_wide(k->mode, a, s);
 }
 
 cudaError_t run_kernel_ordered(const cht::OpArgs& a, void* ctx, cudaStream_t s) {
