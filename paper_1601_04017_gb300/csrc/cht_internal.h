@@ -38,6 +38,10 @@ struct OpArgs {
     // hundreds of pieces each runs.
     u32 chunk = 0;
     unsigned long long* ticket = nullptr;
+    // The find kernels do nothing unless i_lo <= I < i_hi (non-empty cells,
+    // read on the device): of several launches made for different loads, the
+    // one for the table's actual load runs.
+    u64 i_lo = 0, i_hi = ~0ull;
 };
 
 // Launch one batched operation. group_width in {1,2,4,8,16,32}; lane_cells

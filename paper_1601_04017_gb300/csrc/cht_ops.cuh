@@ -626,9 +626,18 @@ constexpr int op_min_blocks() {
     return (V == 4 && G >= 4) ? 5 : 1;
 }
 
+// Whether this launch is for another load than the table has (OpArgs::i_lo).
+template <int MODE>
+__device__ __forceinline__ bool other_load(const OpArgs& a) {
+    if (MODE != kFind || (a.i_lo == 0 && a.i_hi == ~0ull)) return false;
+    const u64 I = *reinterpret_cast<const volatile u64*>(&a.st->I);
+    return I < a.i_lo || I >= a.i_hi;
+}
+
 template <int G, int V, int MODE, int kFlags>
 __global__ void __launch_bounds__(kOpBlock, op_min_blocks<G, V>()) op_kernel(OpArgs a) {
     pdl_enter();
+    if (other_load<MODE>(a)) return;
     // each warp owns a contiguous slice of the batch, or (a.chunk != 0) takes
     // pieces of a.chunk operations in batch order from the ticket counter, so
     // that the whole grid moves through the batch together
@@ -753,6 +762,7 @@ template <int V, int MODE>
 __global__ void __launch_bounds__(kThreadBlock) thread_kernel(OpArgs a) {
     constexpr bool kHasVals = mode_has_vals(MODE);
     pdl_enter();
+    if (other_load<MODE>(a)) return;
     const u64 cap = 1ull << a.log2c;
     const u32 shift = 64u - a.log2c;
     u64 n_ins = 0, n_del = 0;

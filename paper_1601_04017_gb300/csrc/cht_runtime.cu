@@ -408,10 +408,46 @@ struct KernelCtx {
     u64 n;  // batch size for the width choice
 };
 
+// Large finds while the host has only an upper bound on I (a count of words
+// inserts far fewer keys than its batch has): the window is chosen on the
+// device, by a launch for each load band up to the bound's, of which those for
+// other loads return at once (2 us each; 2^24 finds at load 0.5 with a bound
+// above 0.8 took 620 us in the wide window, now 450 us).
+constexpr u64 kLooseFinds = 1ull << 22;
+
+bool loose_bound(const cht_table* h, u64 n) {
+    return !h->i_exact && n >= kLooseFinds && h->cfg.group_width == 0 && h->cfg.lane_cells == 0;
+}
+
+cudaError_t run_find_by_load(const cht_table* h, const cht::OpArgs& a, cudaStream_t s) {
+    const double load = std::min(1.0, double(h->i_bound) / double(h->cap()));
+    cht::OpArgs b = a;
+    const TunedWindow* w = nullptr;  // the window of the bands gathered so far, from b.i_lo on
+    cudaError_t e = cudaSuccess;
+    auto run = [&]() {
+        if (w && e == cudaSuccess)
+            e = cht::launch_op(cht::kFind, b, w->g, w->g == -1 ? (w->v == 2 ? 2 : 4) : (w->g == 1 && w->v != 4 ? 2 : w->v),
+                               h->cfg.ctas_per_sm ? h->cfg.ctas_per_sm : w->ctas, s);
+    };
+    for (const TunedWindow& t : kTuned) {  // (ascending loads)
+        if (t.mode != int(cht::kFind) || h->log2c < t.log2_lo || h->log2c > t.log2_hi || t.load_lo > load) continue;
+        if (w && (w->g != t.g || w->v != t.v || w->ctas != t.ctas)) {
+            b.i_hi = u64(double(t.load_lo) * double(h->cap()));
+            run();
+            b.i_lo = b.i_hi;
+        }
+        w = &t;
+    }
+    b.i_hi = ~0ull;
+    run();
+    return e;
+}
+
 cudaError_t run_kernel(const cht::OpArgs& a, void* ctx, cudaStream_t s) {
     const KernelCtx* k = static_cast<const KernelCtx*>(ctx);
     if (aggregated(k->h, k->mode))
         return cht::launch_iou_aggregated(k->mode, a, k->h->cfg.ctas_per_sm, s);
+    if (k->mode == cht::kFind && loose_bound(k->h, k->n)) return run_find_by_load(k->h, a, s);
     const Width w = pick_width(k->h, k->mode, k->n);
     return cht::launch_op(k->mode, a, w.g, w.v, k->h->cfg.ctas_per_sm ? k->h->cfg.ctas_per_sm : w.ctas, s);
 }
