@@ -218,6 +218,7 @@ struct cht_table {
     cht_config cfg = default_config();
     u64 i_bound = 0;      // upper bound on the device's I
     bool i_exact = true;  // i_bound equals the device's I
+    bool i_loose = false;  // (not exact) insertOrUpdate batches, mostly updates, count in i_bound
     cudaStream_t last = nullptr;
 
     u64 cap() const { return 1ull << log2c; }
@@ -408,15 +409,16 @@ struct KernelCtx {
     u64 n;  // batch size for the width choice
 };
 
-// Large finds while the host has only an upper bound on I (a count of words
-// inserts far fewer keys than its batch has): the window is chosen on the
-// device, by a launch for each load band up to the bound's, of which those for
-// other loads return at once (2 us each; 2^24 finds at load 0.5 with a bound
+// Large finds while the host's upper bound on I is likely far above it (a count
+// of words inserts far fewer keys than its batch has): the window is chosen on
+// the device, by a launch for each load band up to the bound's, of which those
+// for other loads return at once (5 us each; 2^24 finds at load 0.5 with a bound
 // above 0.8 took 620 us in the wide window, now 450 us).
 constexpr u64 kLooseFinds = 1ull << 22;
 
 bool loose_bound(const cht_table* h, u64 n) {
-    return !h->i_exact && n >= kLooseFinds && h->cfg.group_width == 0 && h->cfg.lane_cells == 0;
+    return !h->i_exact && (h->i_loose || h->i_bound > h->cap()) && n >= kLooseFinds && h->cfg.group_width == 0 &&
+           h->cfg.lane_cells == 0;
 }
 
 cudaError_t run_find_by_load(const cht_table* h, const cht::OpArgs& a, cudaStream_t s) {
@@ -595,6 +597,7 @@ cht_status grow_in_kernel(cht_table* h, cht::Mode mode, const u64* keys, const u
 // the threshold, migrate, repeat.
 cht_status run_modify_host(cht_table* h, cht::Mode mode, const u64* keys, const u64* vals,
                            unsigned char* codes, u64 n, cudaStream_t s) {
+    h->i_loose = (h->i_loose && !h->i_exact) || mode != cht::kInsert;
     if (!h->growable) {
         const cht_status r = launch(h, mode, keys, vals, nullptr, codes, n, s);
         h->i_bound += n;  // after the launch: the width choice projects n itself

@@ -30,10 +30,10 @@ def test_find_results_by_window(cuda_lib, g, v, load, per_warp, with_codes):
     t.set_config(group_width=g, lane_cells=v, ctas_per_sm=1)
     n = torch.cuda.get_device_properties(0).multi_processor_count * 8 * per_warp - 5
     rng = np.random.default_rng(per_warp)
-    q = np.where(rng.random(n) < 0.5, keys[rng.integers(0, live, n)],
-                 W.uniform_keys(n, start=9_000_000, seed=61))
-    q[rng.integers(0, n, 20)] = 0  # a reserved key: code 3, value 0
-    present = np.isin(q, keys)
+    present = rng.random(n) < 0.5
+    q = np.where(present, keys[rng.integers(0, live, n)], W.uniform_keys(n, start=9_000_000, seed=61))
+    none = rng.integers(0, n, 20)
+    q[none], present[none] = 0, False  # a reserved key: code 3, value 0
     out, codes = vals_buf(n + 8), codes_buf(n + 8)
     t.find(to_dev(q), out, codes if with_codes else None)
     got = to_np_u64(out)
