@@ -2,8 +2,8 @@
 
 Runs the single-call autotuner (cht_tune: every probe window -- group width G,
 cells per lane V, resident CTAs per SM -- timed with at least three trials,
-median kept) on tables of 2^20, 2^24, 2^26 and 2^28 cells at loads 0.25, 0.5, 0.7
-and 0.9, for find (a batch of hits and a batch of misses of c/2 operations each, at
+median kept) on tables of 2^20, 2^24, 2^26 and 2^28 cells at loads 0.25, 0.5, 0.7, 0.85
+and 0.92, for find (a batch of hits and a batch of misses of c/2 operations each, at
 most 2^26, ranked by the sum of the two), insert (two batches that end at the load: the fresh keys that fill
 the table from the previous load level to this one, and the keys up to this
 load into an empty table; ranked by the sum of the two), erase and update
@@ -50,8 +50,8 @@ def builtin_window(op: int, load: float):
 # HBM-resident
 SIZES = (20, 24, 26, 28)
 SIZE_RANGES = {20: (0, 22), 24: (23, 24), 26: (25, 26), 28: (27, 40)}
-LOADS = (0.25, 0.5, 0.7, 0.9)       # tuned loads
-BANDS = {0.25: (0.0, 0.375), 0.5: (0.375, 0.6), 0.7: (0.6, 0.8), 0.9: (0.8, 1.01)}
+LOADS = (0.25, 0.5, 0.7, 0.85, 0.92)  # tuned loads
+BANDS = {0.25: (0.0, 0.375), 0.5: (0.375, 0.6), 0.7: (0.6, 0.8), 0.85: (0.8, 0.875), 0.92: (0.875, 1.01)}
 MODE_NAMES = {0: "cht::kFind", 1: "cht::kInsert", 4: "cht::kErase", 5: "cht::kUpdAdd"}
 
 
