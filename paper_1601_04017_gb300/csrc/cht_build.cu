@@ -46,7 +46,7 @@ struct SortSrc {
 
 __device__ __forceinline__ void load_src(const SortSrc& s, u64 i, u64& k, u64& v) {
     if (s.cells) {
-        ld_cell_nc(s.cells + i, k, v);
+        ld_cell_cg(s.cells + i, k, v);
     } else {
         k = s.keys[i];
         v = s.vals[i];
@@ -88,6 +88,7 @@ constexpr int kMaxPasses = 5;  // sort keys of at most 40 bits
 // reserved status bit; they never enter the table.
 __global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const u64* keys, u64 n, u32 B, u32* hist,
                                                                    BuildExtra* ex, int full_keys) {
+    pdl_enter();
     __shared__ u32 bins[kMaxPasses][kDigits];
     const int passes = int(B / 8);
     for (int p = 0; p < passes; ++p) bins[p][threadIdx.x] = 0;
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(PassArgs a)
                 ks[q] = a.src.keys[i];
                 vs[q] = a.src.vals[i];
             } else {
-                ld_cell_nc(a.src.cells + i, ks[q], vs[q]);
+                ld_cell_cg(a.src.cells + i, ks[q], vs[q]);
             }
         }
     }
@@ -311,6 +312,7 @@ constexpr size_t pass_smem_bytes() {
 // exclusive scan of u32 (the digit-major histogram), in place
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const u32* in, u64 m, u32* part) {
+    pdl_enter();
     __shared__ u32 sh[kScanThreads / 32];
     const u64 base = u64(blockIdx.x) * kScanChunk;
     u32 s = 0;
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const u32* in
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_partials_kernel(u32* part, u64 np) {
+    pdl_enter();
     __shared__ u32 sh[kScanThreads / 32];
     u32 carry = 0;
     for (u64 b = 0; b < np; b += kScanThreads) {
@@ -337,6 +340,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_partials_kernel(u32* part, 
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(u32* data, u64 m, const u32* part) {
+    pdl_enter();
     __shared__ u32 sh[kScanThreads / 32];
     const u64 base = u64(blockIdx.x) * kScanChunk;
     u32 carry = part[blockIdx.x];
@@ -352,9 +356,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(u32* data, u64
 
 cudaError_t scan_exclusive(u32* data, u64 m, u32* part, cudaStream_t s) {
     const u64 nb = (m + kScanChunk - 1) / kScanChunk;
-    scan_reduce_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(data, m, part);
-    scan_partials_kernel<<<1, kScanThreads, 0, s>>>(part, nb);
-    scan_apply_kernel<<<unsigned(nb), kScanThreads, 0, s>>>(data, m, part);
+    launch_overlapped(scan_reduce_kernel, unsigned(nb), kScanThreads, 0, s, data, m, part);
+    launch_overlapped(scan_partials_kernel, 1, kScanThreads, 0, s, part, nb);
+    launch_overlapped(scan_apply_kernel, unsigned(nb), kScanThreads, 0, s, data, m, part);
     count_launch();
     count_launch();
     count_launch();
@@ -419,9 +423,11 @@ struct PlaceArgs {
     BuildExtra* ex;
 };
 
+// (These kernels overlap the launches before them, which write what they read:
+// their loads are coherent ones, not read-only ones.)
 __device__ __forceinline__ u64 ld_key(const Cell* p) {
     u64 k;
-    asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(k) : "l"(p));
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(k) : "l"(p));
     return k;
 }
 
@@ -468,6 +474,7 @@ constexpr u32 kPlacePad = kPlaceChunk + kPlaceChunk / kPlaceItems;
 
 template <int MODE>
 __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
+    pdl_enter();
     __shared__ u32 shc[8];
     __shared__ long long shm[8];
     __shared__ u32 ic[256];
@@ -492,7 +499,7 @@ __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
             k[q] = kEmpty;
             v[q] = 0;
             if (i < a.n) {
-                if (MODE == 2) ld_cell_nc(a.srt + i, k[q], v[q]);
+                if (MODE == 2) ld_cell_cg(a.srt + i, k[q], v[q]);
                 else k[q] = ld_key(a.srt + i);
             }
         }
@@ -640,6 +647,7 @@ u64 place_smem_bytes() {
 // marks its chunk for the recount.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) build_resolve_kernel(PlaceArgs a) {
+    pdl_enter();
     __shared__ u64 sh_found[8], sh_end[8];
     const u32 nd = a.ex->n_deferred;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -698,6 +706,7 @@ __global__ void __launch_bounds__(256) build_resolve_kernel(PlaceArgs a) {
 constexpr u32 kScanJoins = 2048;
 
 __global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 np, BuildExtra* ex) {
+    pdl_enter();
     __shared__ Agg st[kScanJoins / 8 * 9];
     __shared__ u32 shc[8];
     __shared__ long long shm[8];
@@ -763,6 +772,7 @@ __global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 n
 // special slots (the last copy's value).
 __global__ void build_finish_kernel(Cell* cells, u32 log2c, const Cell* ov, BuildExtra* ex, DevState* st,
                                     const u64* vals) {
+    pdl_enter();
     if (threadIdx.x != 0) return;
     const u64 c = 1ull << log2c;
     const u64 S = ex->S;
@@ -870,11 +880,13 @@ __device__ __forceinline__ u64 merge_split(const MergeArgs& a, u64 diag) {
 }
 
 __global__ void __launch_bounds__(128) merge_split_kernel(MergeArgs a) {
+    pdl_enter();
     const u64 tot = a.nx + a.ny, t = u64(blockIdx.x) * 128 + threadIdx.x, d = t * kPlaceChunk;
     if (d < tot + kPlaceChunk) a.split[t] = u32(merge_split(a, d < tot ? d : tot));
 }
 
 __global__ void __launch_bounds__(256) merge_runs_kernel(MergeArgs a) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char msm[];
     Cell* const stage = reinterpret_cast<Cell*>(msm);            // x's part, then y's
     u64* const sk = reinterpret_cast<u64*>(stage + kPlaceChunk);  // their sort keys
@@ -888,7 +900,7 @@ __global__ void __launch_bounds__(256) merge_runs_kernel(MergeArgs a) {
         const u32 j = u32(q) * 256 + threadIdx.x;
         if (j < m) {
             Cell cl;
-            ld_cell_nc(j < nx ? a.x + x0 + j : a.y + y0 + (j - nx), cl.key, cl.val);
+            ld_cell_cg(j < nx ? a.x + x0 + j : a.y + y0 + (j - nx), cl.key, cl.val);
             stage[j] = cl;
             sk[j] = sort_key(cl.key, a.B);
         }
@@ -932,8 +944,8 @@ cudaError_t launch_build_merge(const Cell* x, u64 nx, const Cell* y, u64 ny, u32
     const u64 tot = nx + ny, tiles = (tot + kPlaceChunk - 1) / kPlaceChunk;
     // (the sort's tile prefixes are not used by a merge: 2 KB per 4096 cells)
     a.split = reinterpret_cast<u32*>(static_cast<unsigned char*>(scratch) + Layout(tot).off_tiles);
-    merge_split_kernel<<<unsigned((tiles + 1 + 127) / 128), 128, 0, s>>>(a);
-    merge_runs_kernel<<<unsigned(tiles), 256, smem, s>>>(a);
+    launch_overlapped(merge_split_kernel, unsigned((tiles + 1 + 127) / 128), 128, 0, s, a);
+    launch_overlapped(merge_runs_kernel, unsigned(tiles), 256, smem, s, a);
     count_launch();
     count_launch();
     *merged = a.out;
@@ -963,7 +975,7 @@ cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c
     if (e != cudaSuccess) return e;
     u64 cgrid = u64(sm_count()) * 8;
     if (cgrid > (n + kSortThreads * 8 - 1) / (kSortThreads * 8)) cgrid = (n + kSortThreads * 8 - 1) / (kSortThreads * 8);
-    radix_count_kernel<<<unsigned(cgrid), kSortThreads, 0, s>>>(keys, n, B, counts, ex, full_keys);
+    launch_overlapped(radix_count_kernel, unsigned(cgrid), kSortThreads, 0, s, keys, n, B, counts, ex, full_keys);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     constexpr size_t smem = pass_smem_bytes();
@@ -983,17 +995,8 @@ cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c
         a.dst = buf[cur];
         a.hist = counts + a.pass * kDigits;
         a.ticket = counts + kMaxPasses * kDigits + a.pass;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(unsigned(L.ntiles));
-        cfg.blockDim = dim3(kPassThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];  // the next pass's launch overlaps this one's tail
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, a.pass == 0 ? radix_pass_kernel<true> : radix_pass_kernel<false>, a);
+        e = launch_overlapped(a.pass == 0 ? radix_pass_kernel<true> : radix_pass_kernel<false>, unsigned(L.ntiles),
+                              kPassThreads, smem, s, a);
         count_launch();
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1011,11 +1014,11 @@ cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scrat
     const PlaceArgs a = place_args(sorted, n, log2c, scratch, ex);
     cudaError_t e = cudaMemsetAsync(a.dirty, 0, L.nchunks, s);
     if (e != cudaSuccess) return e;
-    build_place_kernel<0><<<unsigned(L.nchunks), 256, place_smem_bytes<0>(), s>>>(a);
+    launch_overlapped(build_place_kernel<0>, unsigned(L.nchunks), 256, place_smem_bytes<0>(), s, a);
     // deferred survivor tests (both kernels return at once when there are none)
-    build_resolve_kernel<<<unsigned(sm_count() * 4), 256, 0, s>>>(a);
-    build_place_kernel<1><<<unsigned(L.nchunks), 256, place_smem_bytes<1>(), s>>>(a);
-    build_place_scan_kernel<<<1, 256, 0, s>>>(a.parts, L.nchunks, ex);
+    launch_overlapped(build_resolve_kernel, unsigned(sm_count() * 4), 256, 0, s, a);
+    launch_overlapped(build_place_kernel<1>, unsigned(L.nchunks), 256, place_smem_bytes<1>(), s, a);
+    launch_overlapped(build_place_scan_kernel, 1, 256, 0, s, a.parts, L.nchunks, ex);
     for (int i = 0; i < 4; ++i) count_launch();
     return cudaGetLastError();
 }
@@ -1037,8 +1040,8 @@ cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c
     cudaError_t e = cudaFuncSetAttribute(build_place_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(place_smem_bytes<2>()));
     if (e != cudaSuccess) return e;
-    build_place_kernel<2><<<unsigned(L.nchunks), 256, place_smem_bytes<2>(), s>>>(a);
-    build_finish_kernel<<<1, 32, 0, s>>>(cells, log2c, a.ov, ex, st, vals);
+    launch_overlapped(build_place_kernel<2>, unsigned(L.nchunks), 256, place_smem_bytes<2>(), s, a);
+    launch_overlapped(build_finish_kernel, 1, 32, 0, s, cells, log2c, a.ov, ex, st, vals);
     count_launch();
     count_launch();
     return cudaGetLastError();

@@ -244,6 +244,7 @@ constexpr int kMaxTombWalk = 32;  // tombstones a live cell looks back over
 template <bool kCheck>
 __global__ void __launch_bounds__(kPThreads) live_count_kernel(const Cell* cells, u32 log2c, u32 B, u32* counts,
                                                                u32* unsorted) {
+    pdl_enter();
     __shared__ u32 wsum[kPWarps];
     const u64 c = 1ull << log2c;
     const u64 base = u64(blockIdx.x) * kCompactChunk;
@@ -295,8 +296,9 @@ __global__ void __launch_bounds__(kPThreads) live_count_kernel(const Cell* cells
 
 // A warp keeps its 16 windows' cells in registers between counting and writing
 // them: the table is read once.
-__global__ void __launch_bounds__(kPThreads) live_write_kernel(const Cell* cells, u64 c, const u32* offs,
+__global__ void __launch_bounds__(kPThreads, 3) live_write_kernel(const Cell* cells, u64 c, const u32* offs,
                                                                u64* keys_out, u64* vals_out, Cell* cells_out) {
+    pdl_enter();
     __shared__ u32 wcount[kPWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const u32 below = (1u << lane) - 1u;
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(kPThreads) live_write_kernel(const Cell* cells
         const u64 i = base + u * 32 + lane;
         k[u] = kEmpty;
         v[u] = 0;
-        if (i < c) ld_cell_nc(cells + i, k[u], v[u]);
+        if (i < c) ld_cell_cg(cells + i, k[u], v[u]);
     }
     u32 cnt = 0;
 #pragma unroll
@@ -491,11 +493,11 @@ cudaError_t launch_compact_count(const Cell* cells, u32 log2c, bool check, void*
     cudaError_t e = cudaMemsetAsync(*unsorted, 0, sizeof(u32), s);
     if (e != cudaSuccess) return e;
     if (check)
-        live_count_kernel<true><<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, log2c, build_sort_bits(log2c), counts,
-                                                                        *unsorted);
+        launch_overlapped(live_count_kernel<true>, unsigned(L.nchunks), kPThreads, 0, s, cells, log2c,
+                          build_sort_bits(log2c), counts, *unsorted);
     else
-        live_count_kernel<false><<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, log2c, build_sort_bits(log2c), counts,
-                                                                         *unsorted);
+        launch_overlapped(live_count_kernel<false>, unsigned(L.nchunks), kPThreads, 0, s, cells, log2c,
+                          build_sort_bits(log2c), counts, *unsorted);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return scan_exclusive_u32(counts, L.nchunks, reinterpret_cast<u32*>(b + L.o_part), s);
@@ -504,8 +506,8 @@ cudaError_t launch_compact_count(const Cell* cells, u32 log2c, bool check, void*
 cudaError_t launch_compact_write(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, Cell* cells_out,
                                  void* scratch, cudaStream_t s) {
     const CompactScratch L(log2c);
-    live_write_kernel<<<unsigned(L.nchunks), kPThreads, 0, s>>>(cells, 1ull << log2c, static_cast<const u32*>(scratch),
-                                                               keys_out, vals_out, cells_out);
+    launch_overlapped(live_write_kernel, unsigned(L.nchunks), kPThreads, 0, s, cells, 1ull << log2c,
+                      static_cast<const u32*>(scratch), keys_out, vals_out, cells_out);
     count_launch();
     return cudaGetLastError();
 }

@@ -44,6 +44,24 @@ struct OpArgs {
     u64 i_lo = 0, i_hi = ~0ull;
 };
 
+// Launch with programmatic stream serialization: the kernel's launch overlaps
+// the tail of the one before it.  Kernels launched so begin with pdl_enter.
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                              A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Launch one batched operation. group_width in {1,2,4,8,16,32}; lane_cells
 // 1 or 2 (G = 1 always uses 2; G = 32 only 1); ctas_per_sm 0 = occupancy
 // maximum.  Returns the launch error (cudaSuccess if none).

@@ -299,20 +299,9 @@ cudaError_t launch_shrink(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log2
 
 namespace {
 
-// Launch with programmatic stream serialization (see pdl_enter).
 template <typename K>
-cudaError_t launch_pdl(K kernel, unsigned grid, size_t smem, cudaStream_t s, const MigArgs& a) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kMigBlock);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+cudaError_t launch_counted(K kernel, unsigned grid, size_t smem, cudaStream_t s, const MigArgs& a) {
+    const cudaError_t e = launch_overlapped(kernel, grid, kMigBlock, smem, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -361,10 +350,10 @@ cudaError_t launch_migrate(const Cell* src, u32 src_log2, Cell* dst, u32 dst_log
     u64 grid = u64(sm_count()) * per_sm;
     const u64 need = (ntiles + kMigWarps - 1) / kMigWarps;
     if (grid > need) grid = need;
-    e = windows ? launch_pdl(migrate_window_kernel, unsigned(grid), smem, s, a)
-                : launch_pdl(migrate_walk_kernel, unsigned(grid), smem, s, a);
+    e = windows ? launch_counted(migrate_window_kernel, unsigned(grid), smem, s, a)
+                : launch_counted(migrate_walk_kernel, unsigned(grid), smem, s, a);
     if (e != cudaSuccess) return e;
-    return launch_pdl(migrate_finish_kernel, 1, 0, s, a);
+    return launch_counted(migrate_finish_kernel, 1, 0, s, a);
 }
 
 cudaError_t launch_export(const Cell* cells, u32 log2c, u64* keys_out, u64* vals_out, u64 max_n,

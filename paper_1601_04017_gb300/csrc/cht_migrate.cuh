@@ -27,14 +27,9 @@ struct MigArgs {
     u32 start_cap;   // per-warp capacity of the cluster-start list (walk kernel)
 };
 
-__device__ __forceinline__ u64 ld_key_nc(const Cell* p) {
-    u64 k;
-    asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(k) : "l"(p));
-    return k;
-}
-
-// Source loads: the read-only path when the source was written before the
-// launch (the migration kernels), L2 only (kCg) when it was written earlier
+// Source loads.  Ordinary ones, cached in L1, when the source was written
+// before the launch (the migration kernels; not read-only ones, as the launch
+// overlaps the one that wrote it); L2 only (kCg) when it was written earlier
 // in the same launch (the persistent growing kernel, whose SMs may hold stale
 // lines of a buffer from an earlier round in their L1).
 template <bool kCg>
@@ -44,17 +39,14 @@ __device__ __forceinline__ u64 src_key(const Cell* p) {
         asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(k) : "l"(p));
         return k;
     }
-    return ld_key_nc(p);
+    u64 k;
+    asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(k) : "l"(p));
+    return k;
 }
 template <bool kCg>
 __device__ __forceinline__ void src_cell(const Cell* p, u64& k, u64& v) {
     if (kCg) ld_cell_cg(p, k, v);
-    else ld_cell_nc(p, k, v);
-}
-template <bool kCg>
-__device__ __forceinline__ void src_pair(const Cell* p, u64& k0, u64& v0, u64& k1, u64& v1) {
-    if (kCg) ld_pair_cg(p, k0, v0, k1, v1);
-    else ld_pair_nc(p, k0, v0, k1, v1);
+    else asm volatile("ld.global.ca.v2.u64 {%0,%1}, [%2];" : "=l"(k), "=l"(v) : "l"(p));
 }
 
 // m(d) of a tile border d: d itself if cell d-1 is empty, else one past the

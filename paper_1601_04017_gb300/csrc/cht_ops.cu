@@ -6,23 +6,6 @@
 namespace cht {
 namespace {
 
-// Launch with programmatic stream serialization (see pdl_enter).
-template <typename K>
-cudaError_t launch_pdl(K kernel, unsigned grid, unsigned block, size_t smem, cudaStream_t s, const OpArgs& a) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
-}
-
-
 // Empties a table: zero cells, zero state.  One launch in the chain of
 // overlapping ones (see pdl_enter) instead of two memsets between them, which
 // break it: clear + insert + find on 2^20 cells 42.2 -> 36.0 us a pass.  Tables
@@ -56,7 +39,7 @@ cudaError_t launch_one(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     const u64 need = (a.n + kOpBlock - 1) / kOpBlock;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_pdl(op_kernel<G, V, MODE, kFlags>, unsigned(grid), kOpBlock, 0, s, a);
+    const cudaError_t e = launch_overlapped(op_kernel<G, V, MODE, kFlags>, unsigned(grid), kOpBlock, 0, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -92,7 +75,7 @@ cudaError_t launch_thread_v(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     else if (need >= grid * kThreadOps) grid *= 4;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_pdl(thread_kernel<V, MODE>, unsigned(grid), kThreadBlock, 0, s, a);
+    const cudaError_t e = launch_overlapped(thread_kernel<V, MODE>, unsigned(grid), kThreadBlock, 0, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -195,7 +178,7 @@ cudaError_t launch_agg(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     const u64 nwin = (a.n + 4 * BLOCK - 1) / (4 * BLOCK);
     if (grid > nwin) grid = nwin;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_pdl(iou_agg_kernel<MODE, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
+    const cudaError_t e = launch_overlapped(iou_agg_kernel<MODE, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -214,7 +197,7 @@ cudaError_t launch_clear(Cell* cells, u32 log2c, DevState* st, cudaStream_t s) {
     u64 grid = ((1ull << log2c) / 2 + 255) / 256;
     const u64 most = u64(sm_count()) * 8;
     if (grid > most) grid = most;
-    const cudaError_t e = launch_pdl(clear_kernel, unsigned(grid), 256, 0, s, a);
+    const cudaError_t e = launch_overlapped(clear_kernel, unsigned(grid), 256, 0, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
