@@ -112,6 +112,14 @@ cudaError_t launch_flagged(const OpArgs& a, int g, int v, int flags, int ctas_pe
     return cudaErrorInvalidValue;
 }
 
+// Up to 2^24 cells the finds of the two windows in use there store each result
+// as it comes: L2 holds all or half of the table, its requests don't bound the
+// finds, and the ring's instructions cost more than it saves (load 0.7, direct
+// against ring: 2^22 finds on 2^22 cells 109 and 116 us, 2^23 on 2^23 164 and
+// 188 us, 2^24 on 2^24 453 and 459 us; from 2^25 cells on the ring wins, see
+// kRingOps).
+constexpr u32 kDirectLog2 = 24;
+
 // (group width G, cells per lane V): G = 1 always loads a whole sector.
 template <int MODE>
 cudaError_t launch_mode(const OpArgs& a, int g, int v, int ctas_per_sm, cudaStream_t s) {
@@ -126,8 +134,14 @@ cudaError_t launch_mode(const OpArgs& a, int g, int v, int ctas_per_sm, cudaStre
     if (flags) return launch_flagged<MODE>(a, g, v, flags, ctas_per_sm, s);
     if (v == 4) {
         switch (g) {
-            case 1: return launch_one<1, 4, MODE>(a, ctas_per_sm, s);
-            case 2: return launch_one<2, 4, MODE>(a, ctas_per_sm, s);
+            case 1:
+                if constexpr (MODE == kFind)
+                    if (a.log2c <= kDirectLog2) return launch_one<1, 4, MODE, kFlagDirect>(a, ctas_per_sm, s);
+                return launch_one<1, 4, MODE>(a, ctas_per_sm, s);
+            case 2:
+                if constexpr (MODE == kFind)
+                    if (a.log2c <= kDirectLog2) return launch_one<2, 4, MODE, kFlagDirect>(a, ctas_per_sm, s);
+                return launch_one<2, 4, MODE>(a, ctas_per_sm, s);
             case 4: return launch_one<4, 4, MODE>(a, ctas_per_sm, s);
             case 8: return launch_one<8, 4, MODE>(a, ctas_per_sm, s);
             default: return cudaErrorInvalidValue;

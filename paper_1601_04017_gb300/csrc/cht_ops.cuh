@@ -188,6 +188,7 @@ __device__ __forceinline__ void op_vout(const OpArgs& a, const WarpStage& sg, u6
 // kFlags: bit 0 = tombstone reuse (insert modes), bit 1 = full key space;
 // compile-time, so a table without them runs the plain probe loop.
 constexpr int kFlagReuse = 1;
+constexpr int kFlagDirect = 4;  // finds: no results ring
 constexpr int kFlagFullKeys = 2;
 
 // Results of finds with one-line windows on HBM-sized tables.  Such a find is
