@@ -112,13 +112,13 @@ cudaError_t launch_flagged(const OpArgs& a, int g, int v, int flags, int ctas_pe
     return cudaErrorInvalidValue;
 }
 
-// Up to 2^24 cells the finds of the two windows in use there store each result
-// as it comes: L2 holds all or half of the table, its requests don't bound the
-// finds, and the ring's instructions cost more than it saves (load 0.7, direct
-// against ring: 2^22 finds on 2^22 cells 109 and 116 us, 2^23 on 2^23 164 and
-// 188 us, 2^24 on 2^24 453 and 459 us; from 2^25 cells on the ring wins, see
-// kRingOps).
-constexpr u32 kDirectLog2 = 24;
+// Up to 2^25 cells the finds of the two windows in use there store each result
+// as it comes: L2 holds a good part of the table, its requests don't bound the
+// finds, and the ring's instructions cost as much as it saves or more (load 0.7,
+// direct against ring: 2^22 finds on 2^22 cells 108 and 116 us, 2^23 on 2^23 165
+// and 188 us, 2^24 on 2^24 442 and 459 us, 2^24 on 2^25 535 and 541 us; for
+// 2^26 cells see kRingOps).
+constexpr u32 kDirectLog2 = 25;
 
 // (group width G, cells per lane V): G = 1 always loads a whole sector.
 template <int MODE>

@@ -1,5 +1,5 @@
 """Finds on tables on both sides of the size up to which results are stored
-directly (2^24 cells) rather than through the warp's ring, for the two windows
+directly (2^25 cells) rather than through the warp's ring, for the two windows
 that have both forms.  Results are whole numbers known from the inputs:
 equality, no tolerance.
 """
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("v", [4])
 @pytest.mark.parametrize("g", [1, 2])
-@pytest.mark.parametrize("log2c,live", [(8, 200), (24, 1 << 16), (25, 1 << 16)])
+@pytest.mark.parametrize("log2c,live", [(8, 200), (24, 1 << 16), (25, 1 << 16), (26, 1 << 16)])
 @pytest.mark.parametrize("n", [1, 255, 50_001])
 def test_find_forms(cuda_lib, g, v, log2c, live, n):
     keys = W.uniform_keys(live, start=3_000_000, seed=67)
