@@ -21,6 +21,7 @@
 
 #include "../../include/cht.h"
 #include "cht_internal.h"
+#include "cht_pieces.h"
 
 using cht::Cell;
 using cht::DevState;
@@ -997,17 +998,11 @@ cht_status cht_get_config(cht_handle h, cht_config* cfg) {
 // kPipeChunk operations are staged whole, as smaller ones are, and only copied
 // and run in pieces.
 // ---------------------------------------------------------------------------
-constexpr u64 kPipeChunk = 1ull << 24;
-constexpr u64 kPipeMin = 1ull << 20;
-constexpr int kPipePieces = 8;
+using cht::kPipeChunk;
+using cht::kPipeMin;
+using cht::kPipePieces;
+using cht::pipe_piece;
 constexpr int kPipeSlots = 3;
-
-// operations of a piece of an n-operation batch
-u64 pipe_piece(u64 n) {
-    const u64 unit = 1ull << 16;
-    const u64 p = (n / kPipePieces + unit - 1) / unit * unit;
-    return p < kPipeChunk ? p : kPipeChunk;
-}
 
 struct PipeSlot {
     u64* keys = nullptr;

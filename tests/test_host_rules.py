@@ -1,0 +1,43 @@
+"""Host rules of the library that need no GPU: headers without CUDA in them,
+compiled here with the host compiler and compared with their plain statement.
+"""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1601_04017_gb300", "csrc")
+
+
+@pytest.fixture
+def run_cpp(tmp_path):
+    def run(source, *args):
+        src, exe = tmp_path / "t.cpp", tmp_path / "t"
+        src.write_text(source)
+        subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+        out = subprocess.run([str(exe), *map(str, args)], check=True, capture_output=True, text=True).stdout
+        return [int(x) for x in out.split()]
+
+    return run
+
+
+def test_pieces_cover_a_batch(run_cpp):
+    # around every multiple of a piece's unit in eighths, where the rounding
+    # turns, and both ends of the range that is staged whole
+    lo, hi = 1 << 20, 1 << 24
+    sizes = sorted({n for k in range(2, 33) for d in range(-9, 10) if lo <= (n := (k << 19) + d) <= hi}
+                   | {lo, hi, 7 * (3 << 16) + 1})
+    pieces = run_cpp("""
+#include <cstdio>
+#include <cstdlib>
+#include "cht_pieces.h"
+int main(int n, char** v) {
+    std::printf("%d\\n", cht::kPipePieces);
+    for (int i = 1; i < n; ++i) std::printf("%llu\\n", (unsigned long long)cht::pipe_piece(std::strtoull(v[i], 0, 10)));
+}
+""", *sizes)
+    most = pieces.pop(0)
+    for n, p in zip(sizes, pieces):
+        assert p % (1 << 16) == 0 and -(-n // p) <= most, (n, p)
+        assert p - n / 8 < 1 << 16, (n, p)  # an eighth, rounded up
