@@ -443,14 +443,14 @@ __device__ __forceinline__ void warp_ops(const OpArgs& a, u64 next, const u64 en
             if (V == 1) {
                 if (!kSkipBeforeFirst || o0 >= first) {
                     if (kModify || kCoherent) ld_cell_cg(p, kk[0], vv[0]);
-                    else ld_cell_nc(p, kk[0], vv[0]);
+                    else ld_cell_l1(p, kk[0], vv[0]);
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < V; j += 2) {
                     if (!kSkipBeforeFirst || o0 + j + 1 >= first) {
                         if (kModify || kCoherent) ld_pair_cg(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
-                        else ld_pair_nc(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
+                        else ld_pair_l1(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
                     }
                 }
             }
@@ -719,7 +719,7 @@ __device__ __forceinline__ unsigned char thread_op(const OpArgs& a, u64 key, u64
         const Cell* p = a.cells + base;
 #pragma unroll
         for (int j = 0; j < V; j += 2) {
-            if (MODE == kFind) ld_pair_nc(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
+            if (MODE == kFind) ld_pair_l1(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
             else ld_pair_cg(p + j, kk[j], vv[j], kk[j + 1], vv[j + 1]);
         }
         int hit = -1;

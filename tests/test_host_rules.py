@@ -2,6 +2,7 @@
 compiled here with the host compiler and compared with their plain statement.
 """
 import os
+import re
 import subprocess
 
 import pytest
@@ -41,3 +42,23 @@ int main(int n, char** v) {
     for n, p in zip(sizes, pieces):
         assert p % (1 << 16) == 0 and -(-n // p) <= most, (n, p)
         assert p - n / 8 < 1 << 16, (n, p)  # an eighth, rounded up
+
+
+def test_read_only_loads_stay_in_ordinary_launches():
+    # ld.global.nc needs data that nothing writes while the kernel lives.  A
+    # kernel that begins with pdl_enter lives before the one ahead of it is
+    # done, so neither it nor device functions (which any kernel may call) load
+    # that way.
+    header = re.compile(r"^(?:__global__|__device__|template)[^;{]*\{", re.M)
+    users = 0
+    for f in sorted(os.listdir(CSRC)):
+        text = open(os.path.join(CSRC, f)).read()
+        starts = [m.start() for m in header.finditer(text)]
+        for b, e in zip(starts, starts[1:] + [len(text)]):
+            body = text[b:e]
+            if re.match(r"__device__ __forceinline__ void ld_\w+_nc\(", body):
+                continue  # the load itself
+            if re.search(r"\bld_\w+_nc\(|\.nc\.|__ldg\(", body):
+                users += 1
+                assert "__global__" in body.split("{")[0] and "pdl_enter" not in body, (f, body[:120])
+    assert users > 0
