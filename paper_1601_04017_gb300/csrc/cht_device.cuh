@@ -31,8 +31,8 @@ constexpr unsigned char kNo = 0, kYes = 1, kCodeFull = 2, kCodeReserved = 3;
 //   status: sticky kFull / kReserved bits.
 //   mig_fail, mig_moved: set by a migration warp that could not bound its
 //   cluster range; live elements the migration has placed so far.  Both are
-//   zero between migrations (the last kernel of one clears them), so no
-//   memset precedes a migration.
+//   zero between migrations (the last step of one clears them, the host if it
+//   was not reached), so no memset precedes a migration.
 //   export_pos: output cursor of the export compaction.
 struct DevState {
     u64 I;

@@ -252,6 +252,13 @@ cht_status read_state(cht_table* h, DevState* out, cudaStream_t s) {
     return cuda_status(cudaStreamSynchronize(s));
 }
 
+// Zeroes what a migration that did not reach its last step may have left in
+// the state: the next one starts from zero (see DevState).
+cudaError_t reset_migration(cht_table* h, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(&h->st->mig_fail, 0, sizeof(h->st->mig_fail), s);
+    return e != cudaSuccess ? e : cudaMemsetAsync(&h->st->mig_moved, 0, sizeof(h->st->mig_moved), s);
+}
+
 // Tables too small to give every warp task slot of the GPU (152 SMs x 5 CTAs
 // x 8 warps = 6080) a tile of the usual size are cut finer, down to 64 cells:
 // a tile is one warp's serial work, and a migration of 2^12..2^20 cells takes
@@ -298,6 +305,7 @@ cht_status do_migrate(cht_table* h, u32 new_log2, u64 live, cudaStream_t s) {
             while (tile > 64 && (h->cap() / u64(tile)) < kMigTasks) tile /= 2;
         }
         e = cht::launch_migrate(h->cells, h->log2c, dst, new_log2, h->st, tile, windows, s);
+        if (e != cudaSuccess) reset_migration(h, s);
     }
     if (e != cudaSuccess) {
         lib_free(dst, bytes, s);
@@ -582,7 +590,11 @@ cht_status grow_in_kernel(cht_table* h, cht::Mode mode, const u64* keys, const u
     release();
     h->i_bound = ds.I;
     h->i_exact = true;
-    if (fin.error & cht::kGrowTimeout) return CHT_ERR_TIMEOUT;
+    if (fin.error & cht::kGrowTimeout) {
+        // (the wait may have run out in the middle of a migration)
+        e = reset_migration(h, s);
+        return e != cudaSuccess ? cuda_status(e) : CHT_ERR_TIMEOUT;
+    }
     if (fin.error) {
         // a migration tile could not bound its cluster (or the targets were too
         // small): the host-driven policy, whose migration has a fallback,
