@@ -32,9 +32,8 @@
 // table, or a cluster longer than that) sets mig_fail; a single-CTA kernel,
 // always launched after the tile kernel, sets the counters and, if mig_fail
 // is set, first redoes the whole migration sequentially.
-#include <atomic>
-
 #include "cht_migrate.cuh"
+#include "cht_per_device.h"
 
 namespace cht {
 namespace {
@@ -307,22 +306,21 @@ cudaError_t launch_counted(K kernel, unsigned grid, size_t smem, cudaStream_t s,
 }
 
 // Resident CTAs per SM of a migration kernel with its shared memory for
-// `start_cap` (asked once per kernel and tile size, not per migration).
+// `start_cap` (asked once per device, kernel and tile size, not per migration).
 cudaError_t resident_ctas(bool windows, u32 tile_log2, size_t smem, int* per_sm) {
-    static std::atomic<int> known[2][16];
-    std::atomic<int>& k = known[windows ? 1 : 0][tile_log2 & 15u];
-    *per_sm = k.load(std::memory_order_relaxed);
-    if (*per_sm > 0) return cudaSuccess;
-    const void* fn = windows ? reinterpret_cast<const void*>(migrate_window_kernel)
-                             : reinterpret_cast<const void*>(migrate_walk_kernel);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(migrate_smem_bytes(migrate_start_cap(8192, windows))));
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, kMigBlock, smem);
-    if (e != cudaSuccess) return e;
-    if (*per_sm < 1) *per_sm = 1;
-    k.store(*per_sm, std::memory_order_relaxed);
-    return cudaSuccess;
+    static PerDevice known[2][16];
+    int dev = 0;
+    const cudaError_t e0 = cudaGetDevice(&dev);
+    if (e0 != cudaSuccess) return e0;
+    return known[windows ? 1 : 0][tile_log2 & 15u].get(dev, per_sm, [&](int* n) {
+        const void* fn = windows ? reinterpret_cast<const void*>(migrate_window_kernel)
+                                 : reinterpret_cast<const void*>(migrate_walk_kernel);
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(migrate_smem_bytes(migrate_start_cap(8192, windows))));
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, fn, kMigBlock, smem);
+        if (*n < 1) *n = 1;
+        return e;
+    });
 }
 
 }  // namespace

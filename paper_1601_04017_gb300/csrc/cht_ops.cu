@@ -2,6 +2,7 @@
 #include <atomic>
 
 #include "cht_ops.cuh"
+#include "cht_per_device.h"
 
 namespace cht {
 namespace {
@@ -171,28 +172,27 @@ cudaError_t launch_mode(const OpArgs& a, int g, int v, int ctas_per_sm, cudaStre
 template <int MODE, bool RE, int BLOCK = kAggBlock>
 cudaError_t launch_agg(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     constexpr size_t smem = agg_smem_bytes<MODE, BLOCK>();
-    static std::atomic<int> occ{0};
-    int per_sm = occ.load(std::memory_order_relaxed);
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(iou_agg_kernel<MODE, RE, BLOCK>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
+    static PerDevice known;
+    int dev = 0, per_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = known.get(dev, &per_sm, [&](int* n) {
+        const auto fn = iou_agg_kernel<MODE, RE, BLOCK>;
+        cudaError_t q = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         // as much of the unified L1 / shared memory as shared memory as the
         // kernel can use (38 KB per 256-thread CTA, 152 KB per 1024-thread CTA)
-        e = cudaFuncSetAttribute(iou_agg_kernel<MODE, RE, BLOCK>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 100);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, iou_agg_kernel<MODE, RE, BLOCK>, BLOCK, smem);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        occ.store(per_sm, std::memory_order_relaxed);
-    }
+        if (q == cudaSuccess) q = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, fn, BLOCK, smem);
+        if (*n < 1) *n = 1;
+        return q;
+    });
+    if (e != cudaSuccess) return e;
     if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
     u64 grid = u64(sm_count()) * u64(per_sm);
     const u64 nwin = (a.n + 4 * BLOCK - 1) / (4 * BLOCK);
     if (grid > nwin) grid = nwin;
     if (grid < 1) grid = 1;
-    const cudaError_t e = launch_overlapped(iou_agg_kernel<MODE, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
+    e = launch_overlapped(iou_agg_kernel<MODE, RE, BLOCK>, unsigned(grid), BLOCK, smem, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

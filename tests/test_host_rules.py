@@ -62,3 +62,28 @@ def test_read_only_loads_stay_in_ordinary_launches():
                 users += 1
                 assert "__global__" in body.split("{")[0] and "pdl_enter" not in body, (f, body[:120])
     assert users > 0
+
+
+def test_kept_numbers_are_a_device_s_own(run_cpp):
+    # a kernel attribute set on one device is not set on another: what a launch
+    # needs is asked (and done) on each device it comes to, once
+    got = run_cpp("""
+#include <cstdio>
+#include <initializer_list>
+#include "cht_per_device.h"
+int main() {
+    static cht::PerDevice kept;
+    int fail = 7;
+    for (int dev : {0, 1, 0, 1, 63, 63, 64, 64, 2, 2}) {
+        int asked = 0, n = -1;
+        const int e = kept.get(dev, &n, [&](int* out) {
+            asked = 1;
+            *out = dev + 10;
+            if (dev == 2 && fail) { const int f = fail; fail = 0; return f; }
+            return 0;
+        });
+        std::printf("%d %d %d\\n", e, n, asked);
+    }
+}
+""")
+    assert got == [0, 10, 1, 0, 11, 1, 0, 10, 0, 0, 11, 0, 0, 73, 1, 0, 73, 0, 0, 74, 1, 0, 74, 1, 7, 12, 1, 0, 12, 1]
