@@ -381,6 +381,22 @@ __device__ __forceinline__ Agg agg_join(Agg a, Agg b) {
     return r;
 }
 
+// One past the position of the last survivor (0: none).
+__device__ __forceinline__ u64 agg_end(Agg a) { return a.c ? u64((long long)a.c + a.m) : 0; }
+
+// The cells of a dense write from w0 on that are too many for one CTA: written
+// densely, 2048 at a time behind barriers, they go at a CTA's own rate.  With
+// mostly distinct keys a chunk of 2048 sorted cells owns at most 16 times as
+// many (build_place_dense); copies of few keys leave few survivors and long
+// ranges, which the whole grid zeroes first (build_zero_kernel), and the chunk
+// then writes its survivors alone.  (2^24 copies of 16 keys merged into an
+// empty table of 2^25 cells: 2.88 -> 1.29 ms, 2^24 distinct ones 1.27 ms; the
+// launch that finds nothing to zero costs a merge 2-4 us.)
+constexpr u64 kMaxDense = 1ull << 16;
+struct LongRange {
+    u64 first, count;
+};
+
 // Inclusive scan of one Agg per thread over a 256-thread block; `total` gets
 // the block's join.
 __device__ __forceinline__ Agg block_incl_agg(Agg x, Agg& total, u32* shc, long long* shm) {
@@ -419,6 +435,7 @@ struct PlaceArgs {
     unsigned char* dirty;  // per chunk: a deferred cell of it turned out to survive
     Cell* cells;           // the table
     int dense;             // write every cell of the table, empty ones too
+    LongRange* longs;      // dense: the ranges over kMaxDense (count in ex->n_long)
     Cell* ov;              // survivors past the last cell, by rank
     BuildExtra* ex;
 };
@@ -597,10 +614,16 @@ __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
         const Agg x = {1u, (long long)home};
         carry = agg_join(carry, x);
     }
+    // the cells a dense write covers: from after the last survivor of the chunks
+    // before to this chunk's last one (the last chunk: to the end of the table)
+    u64 w0 = agg_end(first);
+    u64 end = tot.c ? agg_end(agg_join(first, tot)) : w0;
+    if (blockIdx.x + 1 == gridDim.x || end > c) end = c;
+    const bool dense = a.dense && (end <= w0 || end - w0 <= kMaxDense);
     __syncthreads();
     for (u32 j = threadIdx.x; j < tot.c; j += 256) {
         const u64 p = spos[j];
-        if (p < c && a.dense) continue;
+        if (p < c && dense) continue;
         const Cell cl = stage[sidx[j]];
         if (p < c) {
             a.cells[p] = cl;
@@ -610,15 +633,10 @@ __global__ void __launch_bounds__(256) build_place_kernel(PlaceArgs a) {
             atomicMin(&a.ex->first_ov, rank);
         }
     }
-    if (!a.dense) return;
-    // dense: the cells from after the last survivor of the chunks before to
-    // this chunk's last one (the last chunk: to the end of the table), a
-    // window of kPlaceWin cells at a time through a map from cell to survivor
+    if (!dense) return;
+    // dense: a window of kPlaceWin cells at a time through a map from cell to
+    // survivor
     unsigned short* const map = sidx + kPlaceChunk;
-    const bool last = blockIdx.x + 1 == gridDim.x;
-    u64 w0 = first.c ? u64((long long)first.c + first.m) : 0;
-    u64 end = tot.c ? spos[tot.c - 1] + 1 : w0;
-    if (last || end > c) end = c;
     const Cell zero = {0ull, 0ull};
     u32 j = threadIdx.x;  // this thread's next survivor
     for (; w0 < end; w0 += kPlaceWin) {
@@ -705,7 +723,10 @@ __global__ void __launch_bounds__(256) build_resolve_kernel(PlaceArgs a) {
 // took 69 us for 2^14 chunks, 8192 at a time by 1024 threads 30 us.)
 constexpr u32 kScanJoins = 2048;
 
-__global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 np, BuildExtra* ex) {
+// With `longs` (a dense write follows) it also lists the chunks' ranges over
+// kMaxDense, as the write pass computes them.
+__global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 np, BuildExtra* ex, LongRange* longs,
+                                                               u64 c) {
     pdl_enter();
     __shared__ Agg st[kScanJoins / 8 * 9];
     __shared__ u32 shc[8];
@@ -752,6 +773,16 @@ __global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 n
             mine[q] = pre;
             pre = agg_join(pre, y);
         }
+        if (longs) {  // (the thread's eight ranges together, then each)
+            const u64 j0 = b + u64(threadIdx.x) * 8;
+            if (j0 < np && (j0 + 8 >= np || agg_end(pre) > agg_end(mine[0]) + kMaxDense)) {
+                for (u32 q = 0; q < 8 && j0 + q < np; ++q) {
+                    const u64 w0 = agg_end(mine[q]), e1 = agg_end(q < 7 ? mine[q + 1] : pre);
+                    const u64 e = j0 + q + 1 == np || e1 > c ? c : e1;
+                    if (e > w0 && e - w0 > kMaxDense) longs[atomicAdd(&ex->n_long, 1u)] = LongRange{w0, e - w0};
+                }
+            }
+        }
         __syncthreads();
 #pragma unroll
         for (u32 q = 0; q < kScanJoins / 256; ++q) {
@@ -763,6 +794,18 @@ __global__ void __launch_bounds__(256) build_place_scan_kernel(Agg* parts, u64 n
     if (threadIdx.x == 0) {
         ex->S = carry.c;
         ex->first_ov = ~0ull;
+    }
+}
+
+// Zeroes the long ranges, the whole grid on each (none: returns at once).
+__global__ void __launch_bounds__(256) build_zero_kernel(Cell* cells, const LongRange* longs, const BuildExtra* ex) {
+    pdl_enter();
+    const u32 n = ex->n_long;
+    const Cell zero = {0ull, 0ull};
+    for (u32 r = 0; r < n; ++r) {
+        const LongRange x = longs[r];
+        for (u64 i = u64(blockIdx.x) * 256 + threadIdx.x; i < x.count; i += u64(gridDim.x) * 256)
+            cells[x.first + i] = zero;
     }
 }
 
@@ -804,11 +847,11 @@ u32 build_sort_bits(u32 log2c) { return log2c <= 32 ? 32u : 8u * ((log2c + 7u) /
 
 namespace {
 // Scratch layout: two sort buffers, the tiles' digit prefixes, the chunk joins, the survivor flags, the deferred list, the
-// chunks' recount marks, the counters.
+// chunks' recount marks, the long ranges, the counters.
 constexpr u64 kCountBytes = (kMaxPasses * (kDigits + 1) * 4 + 255) & ~255ull;
 struct Layout {
     u64 ntiles, nchunks;
-    u64 off_buf1, off_tiles, off_parts, off_flags, off_def, off_dirty, off_ex, off_counts, total;
+    u64 off_buf1, off_tiles, off_parts, off_flags, off_def, off_dirty, off_long, off_ex, off_counts, total;
     explicit Layout(u64 n) {
         auto al = [](u64 x) { return (x + 255) & ~255ull; };
         ntiles = (n + kSortTile - 1) / kSortTile;
@@ -819,7 +862,9 @@ struct Layout {
         off_flags = off_parts + al(nchunks * sizeof(Agg));
         off_def = off_flags + al(n);
         off_dirty = off_def + al(n * 4);
-        off_ex = off_dirty + al(nchunks);
+        // (a dense write has n >= c / 8: at most c / kMaxDense long ranges)
+        off_long = off_dirty + al(nchunks);
+        off_ex = off_long + al((8 * n / kMaxDense + 2) * sizeof(LongRange));
         off_counts = off_ex + al(sizeof(BuildExtra));  // digit counts and tile tickets of the passes
         total = off_counts + kCountBytes;
     }
@@ -839,6 +884,7 @@ PlaceArgs place_args(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildE
     a.dirty = base + L.off_dirty;
     a.cells = nullptr;
     a.dense = 0;
+    a.longs = reinterpret_cast<LongRange*>(base + L.off_long);
     // the survivors past the last cell go to whichever sort buffer does not
     // hold the sorted cells
     Cell* b0 = reinterpret_cast<Cell*>(base);
@@ -1008,7 +1054,7 @@ cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c
     return cudaSuccess;
 }
 
-cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildExtra* ex,
+cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, bool dense, void* scratch, BuildExtra* ex,
                                cudaStream_t s) {
     const Layout L(n);
     const PlaceArgs a = place_args(sorted, n, log2c, scratch, ex);
@@ -1018,7 +1064,8 @@ cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scrat
     // deferred survivor tests (both kernels return at once when there are none)
     launch_overlapped(build_resolve_kernel, unsigned(sm_count() * 4), 256, 0, s, a);
     launch_overlapped(build_place_kernel<1>, unsigned(L.nchunks), 256, place_smem_bytes<1>(), s, a);
-    launch_overlapped(build_place_scan_kernel, 1, 256, 0, s, a.parts, L.nchunks, ex);
+    launch_overlapped(build_place_scan_kernel, 1, 256, 0, s, a.parts, L.nchunks, ex,
+                      dense && (1ull << log2c) > kMaxDense ? a.longs : nullptr, 1ull << log2c);
     for (int i = 0; i < 4; ++i) count_launch();
     return cudaGetLastError();
 }
@@ -1026,9 +1073,10 @@ cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scrat
 // New cells are written dense by a batch of at least an eighth of their
 // number: whole sectors, empty cells included, so they need not be zeroed
 // first (a merge of 2^25 + 2^22 pairs into 2^26 cells: 160 us of zeroing and a
-// 313 us write, against one of 310 us).  Below that one chunk's range
-// grows past what a CTA should write.  Cells that are zero already take the
-// survivors alone.
+// 313 us write, against one of 310 us).  Below that the ranges of most chunks
+// grow past what a CTA should write; the batch's size stands for its
+// distinct keys here, and chunks with too few of them are told by their range
+// (kMaxDense).  Cells that are zero already take the survivors alone.
 bool build_place_dense(u64 n, u32 log2c) { return n >= (1ull << log2c) / 8; }
 
 cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, bool dense, void* scratch,
@@ -1040,6 +1088,10 @@ cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c
     cudaError_t e = cudaFuncSetAttribute(build_place_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(place_smem_bytes<2>()));
     if (e != cudaSuccess) return e;
+    if (dense && (1ull << log2c) > kMaxDense) {
+        launch_overlapped(build_zero_kernel, unsigned(sm_count()), 256, 0, s, cells, a.longs, ex);
+        count_launch();
+    }
     launch_overlapped(build_place_kernel<2>, unsigned(L.nchunks), 256, place_smem_bytes<2>(), s, a);
     launch_overlapped(build_finish_kernel, 1, 32, 0, s, cells, log2c, a.ov, ex, st, vals);
     count_launch();

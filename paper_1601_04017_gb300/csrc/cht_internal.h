@@ -108,13 +108,13 @@ struct BuildExtra {
     u64 first_ov;    // lowest rank placed past the last cell (~0: none)
     u64 reserved;    // nonzero: a key 0 / ~0 was skipped (full key space off)
     u32 n_deferred;  // cells whose survivor test was deferred to a CTA scan
-    u32 pad;
+    u32 n_long;      // ranges of a dense write that are zeroed first
 };
 u32 build_sort_bits(u32 log2c);
 u64 build_scratch_bytes(u64 n);
 cudaError_t launch_build_sort(const u64* keys, const u64* vals, u64 n, u32 log2c, int full_keys, void* scratch,
                               const Cell** sorted, BuildExtra** ex, cudaStream_t s);
-cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, void* scratch, BuildExtra* ex,
+cudaError_t launch_build_count(const Cell* sorted, u64 n, u32 log2c, bool dense, void* scratch, BuildExtra* ex,
                                cudaStream_t s);
 cudaError_t launch_build_place(const Cell* sorted, u64 n, Cell* cells, u32 log2c, bool dense, void* scratch,
                                BuildExtra* ex, DevState* st, const u64* vals, cudaStream_t s);

@@ -1338,7 +1338,7 @@ cht_status cht_build(cht_handle h, const uint64_t* keys, const uint64_t* vals, u
     cht::BuildExtra* ex = nullptr;
     cudaError_t e = cht::launch_build_sort(static_cast<const u64*>(dk), static_cast<const u64*>(dv), n, h->log2c,
                                            h->cfg.full_key_space, scratch, &sorted, &ex, s);
-    if (e == cudaSuccess) e = cht::launch_build_count(sorted, n, h->log2c, scratch, ex, s);
+    if (e == cudaSuccess) e = cht::launch_build_count(sorted, n, h->log2c, false, scratch, ex, s);
     if (e == cudaSuccess && n >= h->cap()) {
         // only a batch of >= c elements can leave no empty cell: read the
         // survivor count before touching the table
@@ -1447,7 +1447,7 @@ cht_status cht_merge(cht_handle h, const uint64_t* keys, const uint64_t* vals, u
             e = cht::launch_build_sort(ck, cv, tot, nl, h->cfg.full_key_space, bld, &sorted, &ex, s);
         xvals = cv;
     }
-    if (e == cudaSuccess) e = cht::launch_build_count(sorted, tot, nl, bld, ex, s);
+    if (e == cudaSuccess) e = cht::launch_build_count(sorted, tot, nl, dense, bld, ex, s);
     if (e == cudaSuccess && tot >= ncap) {
         // only tot >= c' can leave no empty cell: check before touching the table
         u64 S = 0;
