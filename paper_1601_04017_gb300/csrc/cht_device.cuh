@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "cht_hash.h"
+
 namespace cht {
 
 typedef unsigned long long u64;
@@ -46,16 +48,6 @@ struct DevState {
     u32 sp_present[2];
     u64 mig_moved;
 };
-
-// fmix64, the 64-bit finalizer of MurmurHash3 (Appleby, public domain).
-__device__ __forceinline__ u64 fmix64(u64 x) {
-    x ^= x >> 33;
-    x *= 0xff51afd7ed558ccdull;
-    x ^= x >> 33;
-    x *= 0xc4ceb9fe1a85ec53ull;
-    x ^= x >> 33;
-    return x;
-}
 
 // Scaling map h_c(x) = floor(h(x) * c / 2^64) for c = 2^log2c (Sec. 4.3.1):
 // the top log2c bits.  `shift` is 64 - log2c.

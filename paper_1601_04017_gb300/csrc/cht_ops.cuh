@@ -911,12 +911,6 @@ __device__ __forceinline__ unsigned char global_modify(const OpArgs& a, u64 key,
     return kCodeFull;
 }
 
-// A slot for a key: any mixing of its bits will do (keys need not be random).
-__device__ __forceinline__ u32 slot_hash(u64 k) {
-    const u32 x = (u32(k) ^ u32(k >> 32) * 0x85ebca6bu) * 0x9e3779b1u;
-    return x ^ (x >> 15);
-}
-
 // Shared memory of the aggregation kernel: slot keys, values and first ops;
 // for update modes also each operation's slot and each slot's result (every
 // operation on a key reports whether the key was present).
@@ -1115,7 +1109,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) iou_agg_kernel(OpArgs a) 
         for (int j = 0; j < kPer; ++j) {
             if (!((valid >> j) & 1u)) continue;
             const u64 key = wk[j];
-            u32 s = slot_hash(key) & (kS - 1);
+            u32 s = slot_hash(key, kS - 1);
             bool mine = false;
             for (;;) {
                 u64 k = *reinterpret_cast<volatile u64*>(skey + s);

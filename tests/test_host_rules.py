@@ -87,3 +87,45 @@ int main() {
 }
 """)
     assert got == [0, 10, 1, 0, 11, 1, 0, 10, 0, 0, 11, 0, 0, 73, 1, 0, 73, 0, 0, 74, 1, 0, 74, 1, 7, 12, 1, 0, 12, 1]
+
+
+def test_slots_spread_structured_keys(run_cpp):
+    # looks of linear probing in 2048 slots for a window of 1024 distinct keys,
+    # in hundredths: 150 for random slots (0.5 (1 + 1 / (1 - 0.5))), a few
+    # hundredths more or less by chance
+    got = run_cpp("""
+#include <cstdio>
+#include <vector>
+#include "cht_hash.h"
+typedef unsigned long long u64;
+static int looks(const std::vector<u64>& keys) {
+    static u64 slot[2048];
+    for (u64& s : slot) s = 0;
+    long n = 0;
+    for (u64 k : keys) {
+        unsigned s = cht::slot_hash(k, 2047);
+        for (++n; slot[s]; ++n) s = (s + 1) & 2047;
+        slot[s] = k;
+    }
+    return int(n * 100 / long(keys.size()));
+}
+int main() {
+    std::vector<u64> k(1024);
+    for (int sh = 0; sh < 54; ++sh)  // ids shifted left; strides of addresses and records
+        for (u64 m : {1ull, 3ull, 7ull, 100ull, 4097ull}) {
+            if (m > 1 && sh > 40) continue;
+            for (u64 i = 0; i < 1024; ++i) k[i] = ((i + 1) * m) << sh;
+            std::printf("%d\\n", looks(k));
+        }
+    for (int hi = 10; hi < 59; ++hi) {  // two ids of 32 values each in one word
+        for (u64 i = 0; i < 1024; ++i) k[i] = (((i >> 5) + 1) << hi) | ((i & 31) + 1);
+        std::printf("%d\\n", looks(k));
+    }
+    // keys of one home in 2^16, as a batch sorted by the hash brings them
+    k.clear();
+    for (u64 x = 1; k.size() < 1024; ++x)
+        if (cht::fmix64(x) >> 52 == 77) k.push_back(x);
+    std::printf("%d\\n", looks(k));
+}
+""")
+    assert len(got) == 54 + 4 * 41 + 49 + 1 and max(got) < 200, max(got)
