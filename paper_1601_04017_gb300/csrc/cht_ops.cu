@@ -1,6 +1,7 @@
 // Launchers of the batched probe kernels (see cht_ops.cuh).
 #include <atomic>
 
+#include "cht_grid.h"
 #include "cht_ops.cuh"
 #include "cht_per_device.h"
 
@@ -45,8 +46,6 @@ cudaError_t launch_one(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-constexpr u64 kThreadOps = 8;
-
 // Per-thread operations (group_width = -1), V = 2 or 4 cells per step.
 template <int V, int MODE>
 cudaError_t launch_thread_v(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
@@ -59,23 +58,8 @@ cudaError_t launch_thread_v(const OpArgs& a, int ctas_per_sm, cudaStream_t s) {
         if (per_sm < 1) per_sm = 1;
         occ.store(per_sm, std::memory_order_relaxed);
     }
-    const u64 need = (a.n + kThreadBlock - 1) / kThreadBlock;
-    const u64 wave = u64(sm_count()) * u64(per_sm);
-    if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
-    u64 grid = u64(sm_count()) * u64(per_sm);
-    // The CTAs of overlapping launches go to the SMs that the launch before
-    // leaves first, so a grid with fewer CTAs than fit crowds on some SMs while
-    // others idle.  Modifying batches of about one wave run one operation per
-    // thread (32 rounds of 2^18 inserts and erases behind a growth to 2^24
-    // cells: 2.45 -> 2.36 ms; a find of that size is 2 % slower so); those with at
-    // least kThreadOps operations per thread are cut four times finer, so that
-    // the SMs share them as they come free (counting 2^26 words, then 2^24 finds:
-    // 2.01 -> 1.57 ms); between the two a finer grid only adds a ragged last wave
-    // (2^19 operations: 35.7 against 37.5 us).
-    if (MODE != kFind && need <= wave + wave / 4) grid = need;
-    else if (need >= grid * kThreadOps) grid *= 4;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
+    const u64 grid =
+        thread_grid((a.n + kThreadBlock - 1) / kThreadBlock, u64(sm_count()), u64(per_sm), ctas_per_sm, MODE != kFind);
     const cudaError_t e = launch_overlapped(thread_kernel<V, MODE>, unsigned(grid), kThreadBlock, 0, s, a);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();

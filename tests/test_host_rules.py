@@ -129,3 +129,26 @@ int main() {
 }
 """)
     assert len(got) == 54 + 4 * 41 + 49 + 1 and max(got) < 200, max(got)
+
+
+def test_grid_keeps_to_the_ctas_asked_for(run_cpp):
+    # (operations in CTAs, CTAs per SM that fit, CTAs per SM asked for, modifies)
+    sms = 152
+    cases = [(need, fit, asked, mod) for need in (0, 1, 100, 151, 153, 608, 1216, 1520, 1521, 7295, 7296, 1 << 18, 1 << 27)
+             for fit in (4, 8) for asked in (0, 1, 3, 4, 8, 20) for mod in (0, 1)]
+    got = run_cpp("""
+#include <cstdio>
+#include <cstdlib>
+#include "cht_grid.h"
+int main(int n, char** v) {
+    for (int i = 1; i + 3 < n; i += 4)
+        std::printf("%llu\\n", (unsigned long long)cht::thread_grid(std::strtoull(v[i], 0, 10), 152, std::atoi(v[i + 1]),
+                                                                   std::atoi(v[i + 2]), std::atoi(v[i + 3])));
+}
+""", *(x for c in cases for x in c))
+    for (need, fit, asked, mod), grid in zip(cases, got, strict=True):
+        assert 1 <= grid <= max(need, 1)
+        if asked:
+            assert grid == max(1, min(need, sms * min(asked, fit))), (need, fit, asked, mod, grid)
+        elif need >= sms * fit:
+            assert grid >= sms * fit  # never fewer than a wave
