@@ -1008,7 +1008,7 @@ cht_status cht_get_config(cht_handle h, cht_config* cfg) {
 // kPipeChunk); calls on one device take the slots one after another (a host
 // lock around the enqueueing, events on the GPU).  Batches of kPipeMin to
 // kPipeChunk operations are staged whole, as smaller ones are, and only copied
-// and run in pieces.
+// and run in pieces, on copy streams of their own (PipeLane).
 // ---------------------------------------------------------------------------
 using cht::kPipeChunk;
 using cht::kPipeMin;
@@ -1028,29 +1028,77 @@ struct PipeSlot {
 
 struct DevPipe {
     std::mutex mu;
-    bool tried = false, ok = false;            // the slots
-    bool streams_tried = false, streams = false;  // what every pipelined call needs
+    bool tried = false, ok = false;
     cudaStream_t cin = nullptr, cout = nullptr;
     cudaEvent_t start = nullptr;  // the work on the caller's stream before a call
-    cudaEvent_t in[kPipePieces] = {}, run[kPipePieces] = {}, out = nullptr;  // of a batch staged whole
     PipeSlot slot[kPipeSlots];
     int next = 0;
 };
 DevPipe g_pipe[64];
 
-bool pipe_streams(DevPipe& P) {
-    if (P.streams_tried) return P.streams;
-    P.streams_tried = true;
-    bool ok = cudaStreamCreateWithFlags(&P.cin, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&P.cout, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&P.out, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 0; i < kPipePieces && ok; ++i)
-        ok = cudaEventCreateWithFlags(&P.in[i], cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&P.run[i], cudaEventDisableTiming) == cudaSuccess;
+// Copy streams and events for one call in pieces at a time.  A device has up
+// to kPipeLanes of them, so that calls on different streams don't wait for each
+// other: a call takes the lane its stream had last (their work is in order
+// anyway) or an idle one, and where there is none it is staged on its own
+// stream alone.
+struct PipeLane {
+    cudaStream_t cin = nullptr, cout = nullptr;
+    cudaEvent_t start = nullptr, out = nullptr;
+    cudaEvent_t in[kPipePieces] = {}, run[kPipePieces] = {};
+    cudaEvent_t done = nullptr;     // the end of the last call's work
+    cudaStream_t last = nullptr;    // the stream it ran on
+    bool made = false, used = false, held = false;
+};
+constexpr int kPipeLanes = 4;
+struct DevLanes {
+    std::mutex mu;
+    PipeLane lane[kPipeLanes];
+};
+DevLanes g_lanes[64];
+
+bool make_lane(PipeLane& L) {
+    const auto event = [](cudaEvent_t* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; };
+    bool ok = (L.cin || cudaStreamCreateWithFlags(&L.cin, cudaStreamNonBlocking) == cudaSuccess) &&
+              (L.cout || cudaStreamCreateWithFlags(&L.cout, cudaStreamNonBlocking) == cudaSuccess);
+    for (cudaEvent_t* e : {&L.start, &L.out, &L.done}) ok = ok && (*e || event(e));
+    for (int i = 0; i < kPipePieces; ++i) ok = ok && (L.in[i] || event(&L.in[i])) && (L.run[i] || event(&L.run[i]));
     if (!ok) cudaGetLastError();
-    P.streams = ok;
+    L.made = ok;
     return ok;
+}
+
+// A lane for a call on s, held until it is given back (null: none is idle).
+PipeLane* take_lane(int dev, cudaStream_t s) {
+    DevLanes& D = g_lanes[dev];
+    std::lock_guard<std::mutex> lk(D.mu);
+    PipeLane* got = nullptr;
+    for (PipeLane& L : D.lane)
+        if (L.used && !L.held && L.last == s) got = &L;
+    if (!got) {
+        // (asking an event is no part of a capture that another thread has open)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        for (PipeLane& L : D.lane) {
+            if (L.held) continue;
+            if (L.used && cudaEventQuery(L.done) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (!L.made && !make_lane(L)) continue;
+            got = &L;
+            break;
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (got) got->held = true;
+    return got;
+}
+
+void give_back(int dev, PipeLane* L, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(g_lanes[dev].mu);
+    L->last = s;
+    L->used = true;
+    L->held = false;
 }
 
 bool pipe_ready(int dev) {
@@ -1058,7 +1106,12 @@ bool pipe_ready(int dev) {
     if (P.tried) return P.ok;
     P.tried = true;
     const u64 per = kPipeChunk * (8 + 8 + 8 + 1);
-    if (!pipe_streams(P)) return false;
+    if (cudaStreamCreateWithFlags(&P.cin, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&P.cout, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&P.start, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     unsigned char* mem = nullptr;
     if (cudaMalloc(&mem, per * kPipeSlots) != cudaSuccess) {
         cudaGetLastError();
@@ -1099,9 +1152,8 @@ cht_status piece_launch(cht_table* h, cht::Mode mode, const u64* keys, const u64
 
 // A batch of kPipeMin .. kPipeChunk operations: device copies of the whole host
 // arrays (as the plain way makes them), copied and run in pieces.
-cht_status pipelined_whole(cht_table* h, cht::Mode mode, const u64* keys, const u64* vals, u64* vout,
+cht_status pipelined_whole(PipeLane& P, cht_table* h, cht::Mode mode, const u64* keys, const u64* vals, u64* vout,
                            unsigned char* codes, u64 n, bool hk, bool hv, bool ho, bool hc, cudaStream_t s, PieceFn fn) {
-    DevPipe& P = g_pipe[h->device];
     u64 *bk = nullptr, *bv = nullptr, *bo = nullptr;
     unsigned char* bc = nullptr;
     cht_status r = CHT_OK;
@@ -1148,6 +1200,7 @@ cht_status pipelined_whole(cht_table* h, cht::Mode mode, const u64* keys, const 
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, P.out, 0);
     }
     ok(e);
+    ok(cudaEventRecord(P.done, s));
     lib_free(bk, n * 8, s);
     lib_free(bv, n * 8, s);
     lib_free(bo, n * 8, s);
@@ -1169,20 +1222,22 @@ cht_status pipelined(cht_table* h, cht::Mode mode, const u64* keys, const u64* v
     // pieces of them only cost launches)
     const bool pageable = std::find(kinds, kinds + 4, 2) != kinds + 4;
     if (!(hk || hv || ho || hc)) return CHT_OK;
-    DevPipe& P = g_pipe[h->device];
     if (n <= kPipeChunk) {
         if (pageable) return CHT_OK;
-        // (a capture keeps the plain way: the copy streams are shared)
+        // (a capture keeps the plain way: the copy streams are no part of it)
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
             cudaGetLastError();
             return CHT_OK;
         }
-        std::lock_guard<std::mutex> lk(P.mu);
-        if (!pipe_streams(P)) return CHT_OK;
+        PipeLane* const lane = take_lane(h->device, s);
+        if (!lane) return CHT_OK;
         *handled = true;
-        return pipelined_whole(h, mode, keys, vals, vout, codes, n, hk, hv, ho, hc, s, fn);
+        const cht_status r = pipelined_whole(*lane, h, mode, keys, vals, vout, codes, n, hk, hv, ho, hc, s, fn);
+        give_back(h->device, lane, s);
+        return r;
     }
+    DevPipe& P = g_pipe[h->device];
     std::lock_guard<std::mutex> lk(P.mu);
     if (!pipe_ready(h->device)) return CHT_OK;
     *handled = true;
