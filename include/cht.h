@@ -30,7 +30,8 @@
  *   operations with pinned arrays, and of more than 2^24 with any, are copied
  *   and run in pieces (an eighth of the batch, at most 2^24; 2^24 with
  *   pageable arrays), so the copies of one piece overlap the kernel of
- *   another; the pieces run in order, one linearization of the batch.  Up to
+ *   another; the pieces run in order, one linearization of the batch.  (Up to
+ *   2^24 operations, arrays of a call that share memory are copied whole.)  Up to
  *   2^24 operations, four calls on different streams can do so at a time
  *   without waiting for each other (further ones are copied whole); above, the
  *   calls of a device take turns at three device slots kept by the library

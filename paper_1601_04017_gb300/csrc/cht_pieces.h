@@ -18,4 +18,12 @@ constexpr uint64_t pipe_piece(uint64_t n) {
     return p < kPipeChunk ? p : kPipeChunk;
 }
 
+// Whether two arrays (nbytes long, null: none) share memory.  Inputs are read
+// before results are written in a batch staged whole; in pieces, the results of
+// one would land in the inputs of another still to be copied.
+inline bool share_memory(const void* a, uint64_t abytes, const void* b, uint64_t bbytes) {
+    const uint64_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && (x < y ? y - x < abytes : x - y < bbytes);
+}
+
 }  // namespace cht

@@ -1224,6 +1224,8 @@ cht_status pipelined(cht_table* h, cht::Mode mode, const u64* keys, const u64* v
     if (!(hk || hv || ho || hc)) return CHT_OK;
     if (n <= kPipeChunk) {
         if (pageable) return CHT_OK;
+        for (const void* in : {keys, vals})
+            if (cht::share_memory(in, n * 8, vout, n * 8) || cht::share_memory(in, n * 8, codes, n)) return CHT_OK;
         // (a capture keeps the plain way: the copy streams are no part of it)
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {

@@ -152,3 +152,24 @@ int main(int n, char** v) {
             assert grid == max(1, min(need, sms * min(asked, fit))), (need, fit, asked, mod, grid)
         elif need >= sms * fit:
             assert grid >= sms * fit  # never fewer than a wave
+
+
+def test_arrays_that_share_memory(run_cpp):
+    # every placement of two short arrays (and none)
+    got = run_cpp("""
+#include <cstdio>
+#include "cht_pieces.h"
+int main() {
+    static char m[16];
+    for (int a = 0; a < 6; ++a)
+        for (int an = 1; an < 6; ++an)
+            for (int b = 0; b < 6; ++b)
+                for (int bn = 1; bn < 6; ++bn) {
+                    bool both = false;
+                    for (int x = 0; x < 16; ++x) both |= x >= a && x < a + an && x >= b && x < b + bn;
+                    std::printf("%d\\n", cht::share_memory(m + a, an, m + b, bn) == both);
+                }
+    std::printf("%d\\n", !cht::share_memory(nullptr, 8, m, 8) && !cht::share_memory(m, 8, nullptr, 8));
+}
+""")
+    assert len(got) == 901 and all(got)
