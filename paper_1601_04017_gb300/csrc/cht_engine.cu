@@ -182,9 +182,15 @@ __device__ __forceinline__ void run_item(const EngineArgs& e, const EngineChunk&
 
 // kAhead: for launches whose time is a table's chain of levels rather than the
 // amount of work -- the next item of a group is loaded while the one before it
-// runs (80 registers, 3 CTAs per SM).  Without it 64 registers let 4 CTAs run,
+// runs (81-87 registers, 2 CTAs per SM).  Without it 64 registers let 4 CTAs run,
 // which throughput needs: 1024 tables, 3.7e8 operations, 11.5 ms against
 // 14.0 ms; on 4000 requests to 64 tables the engine takes 3.57 against 3.03 ms.
+// The bound of 64 makes the in-place forms and those with table options spill
+// up to 44 bytes and is faster all the same (256 tables x 24 rounds / 1024
+// tables x 5 rounds; unbounded -> bounded): in place 4 x 2 cells 1393 -> 1087 /
+// 984 -> 618 us, 16 x 1 3179 -> 3028 / 2001 -> 1653; 4 x 2 with tombstone
+// reuse 1064 -> 1032 / 689 -> 585.  With both options 4 x 2 is mixed: 1124 ->
+// 1203 / 711 -> 633.
 template <int G, int V, bool kStaged, int kEF, bool kAhead>
 __global__ void __launch_bounds__(kOpBlock, kAhead ? 1 : 4) engine_kernel(EngineArgs e) {
     constexpr u32 FULL = 0xffffffffu;

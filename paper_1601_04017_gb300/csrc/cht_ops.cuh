@@ -152,7 +152,7 @@ __device__ __forceinline__ int claim_tomb(Cell* cp, u64 key, u64 d) {
 // refill loop; counters and status bits accumulate into the caller's
 // registers (every lane of the warp must call it).  kCoherent: finds read the
 // table through L2 like the modifying modes (required when the same kernel
-// launch also modifies the table); otherwise finds use the read-only path.
+// launch also modifies the table); otherwise finds may hit in L1.
 // Where a warp takes its keys / values and puts its results: the batch's
 // arrays in global memory, or (kStaged) a per-warp area in shared memory that
 // holds operations [base, base + count) -- the engine fills it with one
@@ -823,8 +823,8 @@ namespace cht {
 // sums are two native 32-bit adds (slot_add).  (With 64-bit sums a warp
 // combined its equal keys with match_any first where a window had few distinct
 // ones: 2^26 operations over 2^24 words, s = 0.5 / 1.0 / 1.25 / 1.5: 3.08 / 2.14
-// / 1.59 / 1.20 ms, now 2.87 / 1.95 /
-// 0.96 / 0.61 ms.  Combining in the warp as well costs 0.4 ms at
+// / 1.59 / 1.20 ms, now 2.88 / 1.95 /
+// 0.97 / 0.61 ms.  Combining in the warp as well costs 0.4 ms at
 // s >= 1.25: the native adds take lanes on one slot at once.  Appending a warp's
 // new slots to the window's list with one add costs 0.2 ms at s = 0.5, and all
 // first looks at the slots ahead of the folding give nothing.)
